@@ -212,11 +212,11 @@ def _anneal(st):
     try:
         out = {}
         if c.get("stepwise"):
-            rows = []
+            seen = []
             while P.pa_anneal_step(ctx):
-                rows.append(P.pa_observables(ctx, len(rows)))
+                seen.append(P.pa_observables(ctx, len(seen)))
             for key in ("E_mean", "E2_mean", "C", "lnQ", "S_f", "rho_s"):
-                out[key] = np.array([r[key] for r in rows])
+                out[key] = np.array([o[key] for o in seen])
         else:
             P.pa_anneal(ctx)
             last = P.pa_observables(ctx, c["n"] - 1)
