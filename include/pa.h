@@ -91,7 +91,8 @@ typedef struct {
     /* real couplings: 1 takes the specified Metropolis rule (spec_expf
      * threshold, Sec. II.B) in every lane instead of the verified guard band
      * of pa_check_accept_band; the decisions, and so every result, are the
-     * same (0: the band where it is verified on the device) */
+     * same (0: the band where it is verified on the device).  Lattices whose
+     * sweeps look up tables of the specified thresholds have no band. */
     int32_t exact_accept;
     /* 1: the replica gather of a resampling step (slot j takes replica
      * parent[j], Sec. II.B) runs as its own launch before the sweeps, which
@@ -202,7 +203,9 @@ int pa_overlap(pa_ctx* a, pa_ctx* b, int64_t* hist);
  * violations (may be NULL): floats where the bracket fails (0 expected; real
  * contexts created on a device with violations take the specified rule in every
  * lane).  max_rel_dev (may be NULL): largest |g / spec_expf(-x) - 1| over
- * 0 < x <= 87.  Each context runs the check once per device and process at
+ * 0 < x <= 87.  Lattices whose thresholds fit in shared memory look the
+ * specified threshold up instead; a context of the others (3D L = 12, 3D
+ * L = 10 with a field) runs the check once per device and process at
  * creation.  PA_ECUDA on a CUDA error (message from pa_last_error(NULL)). */
 int pa_check_accept_band(int64_t* violations, double* max_rel_dev);
 
@@ -245,10 +248,10 @@ int pa_profile(pa_ctx* ctx, int enable);
 int pa_phase_times(pa_ctx* ctx, double* ms, int64_t* n, int64_t* launches);
 
 /* ---------------- batched instances ----------------
- * Many disorder realisations annealed together: one persistent sweep launch
- * covers every instance's replica tiles (mixed L, +-J and real couplings),
- * resampling and observables run as one launch each for all instances, and
- * pa_batch_run captures the schedule into a CUDA graph.  All instances share
+ * Many disorder realisations annealed together: persistent sweep launches
+ * cover every instance's replica tiles (mixed L; one launch for +-J, one
+ * beside it for real couplings), resampling and observables run as one launch
+ * each for all instances, and pa_batch_run captures the schedule into a CUDA graph.  All instances share
  * D, the schedule (betas, n_sweeps) and the Philox key (seed); each has its
  * own rng_instance, so its results are identical to a single-instance
  * context created with the same arguments.  Sweep shapes (groups per block of

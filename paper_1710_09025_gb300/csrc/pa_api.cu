@@ -33,6 +33,7 @@ struct pa_ctx {
     cudaStream_t st;
     int gpb, threads, real_warps;
     int band;                   // real couplings: acceptance guard band verified on this device
+    int field;                  // some h is not zero (after the flush)
     double betaF0, log_R;
     std::vector<double> betas;
     std::vector<int> Rk;        // population (target) at each temperature; R = capacity
@@ -420,6 +421,8 @@ static int create_impl(pa_ctx** out, int D, int L, int kind, const float* J, con
             c->hh[i] = flush73(h[i]);
             nflush += (c->hh[i] != h[i]);
         }
+    c->field = 0;
+    for (int i = 0; i < N; ++i) c->field |= c->hh[i] != 0.0f;
     if (nflush) c->err = "warning: " + std::to_string(nflush) + " coupling/field magnitudes below 2^-73 flushed to 0";
 
     Layout lay = make_layout(D, L, kind, c->layout, cap, n_temps, c->acc_grad, c->shard_total);
@@ -527,7 +530,9 @@ static int create_impl(pa_ctx** out, int D, int L, int kind, const float* J, con
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);  // host vectors above go out of scope
         if (e != cudaSuccess) { g_create_err = cudaGetErrorString(e); rc2 = PA_ECUDA; }
     }
-    c->band = (rc2 == PA_OK && kind == PA_REAL && !o.exact_accept) ? pa::accept_band_ok(c->st) : 0;
+    // the band check (tens of ms once per device and process) only where the sweeps use it
+    c->band = (rc2 == PA_OK && kind == PA_REAL && !o.exact_accept && !pa::real_uses_table(D, L, c->field != 0))
+                  ? pa::accept_band_ok(c->st) : 0;
     if (rc2 != PA_OK) {
         if (c->own_ws) cudaFree(c->ws);
         delete c;
@@ -716,6 +721,7 @@ static void plan_step(pa_ctx* c, StepPlan* pl)
         pa::RealInst& in = pl->re.i;
         in.Sin = c->S8[c->cur]; in.Sout = c->S8[c->cur ^ 1];
         in.parent = k > 0 ? c->parent : nullptr;
+        in.field = c->field;
         in.J = c->J; in.h = c->h; in.Jfix = c->Jfix; in.hfix = c->hfix; in.E = c->E128;
         in.cJ = c->acc_grad ? c->cJ + (size_t)k * c->D * c->N : nullptr;
         in.ch = c->acc_grad ? c->ch + (size_t)k * c->N : nullptr;
@@ -1517,7 +1523,12 @@ struct pa_batch {
     int2* d_items[2];              // work items per groups-per-block multiplier
     int n_items[2];
     size_t smem[2];
-    int* d_counters;               // [n_temps + kTuneSlots]
+    int2* d_titems;                // work items of the threshold-table launch
+    int n_titems, tblocks, tchunk;
+    size_t tsmem;
+    cudaStream_t st2;              // the table launch runs beside the other sweep launch (fork and join by events)
+    cudaEvent_t ev_fork, ev_join;
+    int* d_counters;               // [n_temps + kTuneSlots], then [n_temps] of the table launch
     std::vector<int> after_cur, after_fam;  // [k * n_inst + i]: context state after step k
     int maxR;
     bool has_packed;
@@ -1556,8 +1567,12 @@ static void batch_free(pa_batch* b)
     cudaFree(b->d_ob);
     cudaFree(b->d_items[0]);
     cudaFree(b->d_items[1]);
+    cudaFree(b->d_titems);
     cudaFree(b->d_counters);
     cudaFree(b->ws);
+    if (b->ev_fork) cudaEventDestroy(b->ev_fork);
+    if (b->ev_join) cudaEventDestroy(b->ev_join);
+    if (b->st2) cudaStreamDestroy(b->st2);
     delete b;
 }
 
@@ -1579,7 +1594,9 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
     b->D = D; b->n_inst = n_inst; b->n_temps = n_temps; b->n_sweeps = n_sweeps; b->k_next = 0;
     b->seed = seed; b->st = (cudaStream_t)stream; b->ws = nullptr;
     b->d_rs = nullptr; b->d_sw = nullptr; b->d_ob = nullptr;
-    b->d_items[0] = b->d_items[1] = nullptr; b->d_counters = nullptr; b->gexec = nullptr;
+    b->d_items[0] = b->d_items[1] = b->d_titems = nullptr; b->d_counters = nullptr; b->gexec = nullptr;
+    b->n_items[0] = b->n_items[1] = b->n_titems = b->tblocks = 0; b->tsmem = 0;
+    b->tchunk = pa::kBatchTableGroups; b->st2 = nullptr; b->ev_fork = b->ev_join = nullptr;
     b->tune_mode = (opt && opt->threads < 0) ? -1 : 0;
     b->tuned = b->tune_mode < 0;
     b->blocks = 0; b->mult = 1; b->tune_slot = 0; b->tuned_ms = 0.0; b->launches = 0;
@@ -1597,7 +1614,7 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
         int cls, tiles;
         size_t sm;
         int G = (d.R + 63) / 64;
-        if (rc == PA_OK && !pa::batch_class(D, d.L, d.kind, 1, G, d.R, &cls, &tiles, &sm)) {
+        if (rc == PA_OK && !pa::batch_class(D, d.L, d.kind, false, 1, pa::kBatchTableGroups, G, d.R, &cls, &tiles, &sm)) {
             err = "lattice size not supported by the batched sweep (3D L in 4..12 even or 16)";
             rc = PA_EINVAL;
         }
@@ -1635,7 +1652,7 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
             return rc;
         }
         b->ctx.push_back(c);
-        if (d.kind == PA_REAL) b->band = c->band;  // one verdict per device
+        if (d.kind == PA_REAL && c->band) b->band = c->band;  // one verdict per device
     }
     // argument tables for every (temperature, instance)
     const size_t nt = (size_t)n_temps * n_inst;
@@ -1648,7 +1665,7 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
         pa_ctx* c = b->ctx[i];
         int cls, tiles;
         size_t sm;
-        pa::batch_class(D, c->L, c->kind, 1, c->G, c->R, &cls, &tiles, &sm);
+        pa::batch_class(D, c->L, c->kind, c->field != 0, 1, b->tchunk, c->G, c->R, &cls, &tiles, &sm);
         for (int k = 0; k < n_temps; ++k) {
             StepPlan pl;
             plan_step(c, &pl);
@@ -1668,8 +1685,22 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
         }
         c->k_next = 0; c->cur = 0; c->famcur = 0;
     }
-    // work items, most expensive first (estimated thread-instructions per tile)
-    for (int m = 1; m <= 2; ++m) {
+    // chunks of the threshold-table launch: as large as leaves two per SM (a
+    // chunk builds the instance's table, so small ones cost work; too few leave
+    // SMs idle)
+    int dev = 0, sms = 0, per = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    for (; b->tchunk > pa::kBatchTableLeast; b->tchunk /= 2) {
+        long long n = 0;
+        for (auto* c : b->ctx)
+            if (c->kind == PA_REAL) n += ((c->R + 3) / 4 + b->tchunk - 1) / b->tchunk;
+        if (n >= 2ll * sms) break;
+    }
+    // work items, most expensive first (estimated thread-instructions per
+    // tile): one list for the launch of each groups-per-block multiplier, one
+    // (m = 0) for the threshold-table launch
+    for (int m = 0; m <= 2 && e == cudaSuccess; ++m) {
         struct It { double cost; int inst, tile; };
         std::vector<It> items;
         size_t smax = 0;
@@ -1677,7 +1708,8 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
             pa_ctx* c = b->ctx[i];
             int cls, tiles;
             size_t sm;
-            pa::batch_class(D, c->L, c->kind, m, c->G, c->R, &cls, &tiles, &sm);
+            pa::batch_class(D, c->L, c->kind, c->field != 0, m > 0 ? m : 1, b->tchunk, c->G, c->R, &cls, &tiles, &sm);
+            if ((cls >= pa::kBatchTableBase) != (m == 0)) continue;
             smax = std::max(smax, sm);
             int gpb = 0, thr = 0;
             pa::packed_default_shape(D, c->L, &gpb, &thr);
@@ -1687,32 +1719,50 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
         std::stable_sort(items.begin(), items.end(), [](const It& x, const It& y) { return x.cost > y.cost; });
         std::vector<int2> h(items.size());
         for (size_t t = 0; t < items.size(); ++t) h[t] = make_int2(items[t].inst, items[t].tile);
-        b->n_items[m - 1] = (int)items.size();
-        b->smem[m - 1] = smax;
-        e = cudaMalloc(&b->d_items[m - 1], sizeof(int2) * h.size());
-        if (e == cudaSuccess)
-            e = cudaMemcpy(b->d_items[m - 1], h.data(), sizeof(int2) * h.size(), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) break;
+        int2** d = m == 0 ? &b->d_titems : &b->d_items[m - 1];
+        if (m == 0) { b->n_titems = (int)items.size(); b->tsmem = smax; }
+        else { b->n_items[m - 1] = (int)items.size(); b->smem[m - 1] = smax; }
+        if (items.empty()) continue;
+        e = cudaMalloc(d, sizeof(int2) * h.size());
+        if (e == cudaSuccess) e = cudaMemcpy(*d, h.data(), sizeof(int2) * h.size(), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) e = cudaMalloc(&b->d_rs, sizeof(pa::ResampleArgs) * nt);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_sw, sizeof(pa::BatchSweepInst) * nt);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_ob, sizeof(pa::ObsArgs) * nt);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counters, sizeof(int) * (n_temps + kTuneSlots));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_counters, sizeof(int) * (2 * n_temps + kTuneSlots));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_rs, rs.data(), sizeof(pa::ResampleArgs) * nt, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_sw, sw.data(), sizeof(pa::BatchSweepInst) * nt, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_ob, ob.data(), sizeof(pa::ObsArgs) * nt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(b->d_counters, 0, sizeof(int) * (n_temps + kTuneSlots));
+    if (e == cudaSuccess) e = cudaMemset(b->d_counters, 0, sizeof(int) * (2 * n_temps + kTuneSlots));
     if (e != cudaSuccess) {
         g_create_err = std::string("batch tables: ") + cudaGetErrorString(e);
         batch_free(b);
         return PA_ECUDA;
     }
     // default sweep configuration: groups-per-block x1, as many blocks as fit
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (pa::batch_sweep_occupancy(std::max(b->smem[0], b->smem[1]), &per) != cudaSuccess || per < 1) per = 1;
     b->blocks = sms * per;
+    if (b->n_titems > 0) {
+        per = 0;
+        e = pa::batch_table_occupancy(b->tsmem, &per);
+        if (e != cudaSuccess || per < 1) {
+            g_create_err = std::string("batch table launch: ") + cudaGetErrorString(e);
+            batch_free(b);
+            return PA_ECUDA;
+        }
+        b->tblocks = std::min(sms * per, b->n_titems);
+        if (b->n_items[0] > 0) {
+            e = cudaStreamCreateWithFlags(&b->st2, cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming);
+            if (e != cudaSuccess) {
+                g_create_err = std::string("batch stream: ") + cudaGetErrorString(e);
+                batch_free(b);
+                return PA_ECUDA;
+            }
+        }
+    }
+    if (b->n_items[0] == 0) b->tuned = true;  // nothing to tune
     // signature of the batch for the tuning cache: SM count and class histogram
     std::map<std::pair<int, int>, int> hist;
     for (auto* c : b->ctx) hist[{c->kind, c->L}] += 1;
@@ -1808,11 +1858,31 @@ static int batch_enqueue(pa_batch* b, bool allow_tune)
     pa::PackedStep ps;
     pa::RealStep rs;
     batch_step_params(b, k, &ps, &rs);
-    PB_CK(b, pa::launch_sweep_batched(ps, rs, b->d_sw + (size_t)k * b->n_inst, b->d_items[b->mult - 1],
-                                      b->n_items[b->mult - 1], b->mult, b->d_counters + k, b->blocks,
-                                      b->smem[b->mult - 1], b->st));
+    const pa::BatchSweepInst* tab = b->d_sw + (size_t)k * b->n_inst;
+    // the two sweep launches are independent: the threshold-table one runs on
+    // the batch's second stream between two events
+    cudaStream_t ts = b->st2 ? b->st2 : b->st;
+    if (b->n_titems > 0) {
+        if (b->st2) {
+            PB_CK(b, cudaEventRecord(b->ev_fork, b->st));
+            PB_CK(b, cudaStreamWaitEvent(b->st2, b->ev_fork, 0));
+        }
+        PB_CK(b, pa::launch_sweep_batched_table(rs, tab, b->d_titems, b->n_titems, b->tchunk,
+                                                b->d_counters + b->n_temps + kTuneSlots + k, b->tblocks, b->tsmem,
+                                                ts));
+        b->launches += 1;
+    }
+    if (b->n_items[b->mult - 1] > 0) {
+        PB_CK(b, pa::launch_sweep_batched(ps, rs, tab, b->d_items[b->mult - 1], b->n_items[b->mult - 1], b->mult,
+                                          b->d_counters + k, b->blocks, b->smem[b->mult - 1], b->st));
+        b->launches += 1;
+    }
+    if (b->st2 && b->n_titems > 0) {
+        PB_CK(b, cudaEventRecord(b->ev_join, b->st2));
+        PB_CK(b, cudaStreamWaitEvent(b->st, b->ev_join, 0));
+    }
     PB_CK(b, pa::launch_observe_batched(b->d_ob + (size_t)k * b->n_inst, b->n_inst, b->maxR, b->st));
-    b->launches += 3;
+    b->launches += 2;
     for (int i = 0; i < b->n_inst; ++i) {
         pa_ctx* c = b->ctx[i];
         c->k_next = k + 1;

@@ -6,6 +6,7 @@
 // single-instance kernels, so every instance gets exactly the results of its
 // own context.  Items are ordered by decreasing cost so that the expensive
 // tiles start first and the tail is made of cheap ones.
+#include "pa_real_table.cuh"
 #include "pa_sweep_tiles.cuh"
 
 namespace pa {
@@ -15,7 +16,10 @@ constexpr int kBatchThreads = 256;
 // 3D lattices the batched sweep dispatches to: packed +-J (two groups-per-
 // block choices) and int8 real couplings.
 #define PA_BATCH_PACKED(X) X(0, 4) X(1, 6) X(2, 8) X(3, 10) X(4, 12) X(5, 16)
-#define PA_BATCH_REAL(X) X(0, 4) X(1, 6) X(2, 8) X(3, 10) X(4, 12)
+#define PA_BATCH_REAL(X) X(3, 10) X(4, 12)
+// 3D lattices of the threshold-table launch (index, L, with a field)
+#define PA_BATCH_TABLE(X) \
+    X(0, 4, false) X(1, 6, false) X(2, 8, false) X(3, 10, false) X(4, 4, true) X(5, 6, true) X(6, 8, true)
 
 __global__ void __launch_bounds__(kBatchThreads, 3) sweep_batch_kernel(PackedStep ps, RealStep rs,
                                                                     const BatchSweepInst* insts,
@@ -58,8 +62,44 @@ __global__ void __launch_bounds__(kBatchThreads, 3) sweep_batch_kernel(PackedSte
     }
 }
 
+// Real couplings on threshold tables: blocks take (instance, chunk of at most
+// `chunk` replica groups) items.  A chunk of 256 replicas amortises the
+// instance's table (at most 64 rule evaluations per site against 2560 attempts
+// per site); small batches take smaller chunks so that every SM has one.
+__global__ void __launch_bounds__(kTabThreads) sweep_batch_table_kernel(RealStep rs, const BatchSweepInst* insts,
+                                                                        const int2* items, int n_items, int chunk,
+                                                                        int* counter)
+{
+    extern __shared__ __align__(128) unsigned char smem_bt[];
+    __shared__ int s_item;
+    for (;;) {
+        if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
+        __syncthreads();
+        const int it = s_item;
+        __syncthreads();
+        if (it >= n_items) return;
+        const int2 w = items[it];
+        const BatchSweepInst& bi = insts[w.x];
+        const int R = bi.re.R, G4 = (R + 3) / 4, n = (G4 + chunk - 1) / chunk;
+        const int g0 = (int)((long long)G4 * w.y / n), g1 = (int)((long long)G4 * (w.y + 1) / n);
+        switch (bi.cls) {
+#define XT(idx, l, f)                                                            \
+    case kBatchTableBase + idx:                                                  \
+        static_assert(8 * TabShape<3, l, f>::W >= kBatchTableGroups, "a chunk fits"); \
+        tab_stage_offsets<3, l, f>(smem_bt);                                     \
+        sweep_real_table<3, l, f>(rs, bi.re, R, g0, g1, smem_bt, false);         \
+        break;
+            PA_BATCH_TABLE(XT)
+#undef XT
+            default:
+                break;
+        }
+    }
+}
+
 // class id, tiles and shared memory of an instance in the batched sweep
-bool batch_class(int D, int L, int kind, int mult, int G, int R, int* cls, int* tiles, size_t* smem)
+bool batch_class(int D, int L, int kind, bool field, int mult, int chunk, int G, int R, int* cls, int* tiles,
+                 size_t* smem)
 {
     if (D != 3) return false;
     if (kind == 0) {
@@ -76,6 +116,16 @@ bool batch_class(int D, int L, int kind, int mult, int G, int R, int* cls, int* 
 #undef XP
         return false;
     }
+#define XT(idx, l, f)                                                                         \
+    if (L == l && field == f) {                                                               \
+        static_assert(TabShape<3, l, f>::FITS, "table fits");                                 \
+        *cls = kBatchTableBase + idx;                                                         \
+        *tiles = ((R + 3) / 4 + chunk - 1) / chunk;                                           \
+        *smem = TabShape<3, l, f>::SMEM;                                                      \
+        return true;                                                                          \
+    }
+    PA_BATCH_TABLE(XT)
+#undef XT
 #define XR(idx, l)                                                                            \
     if (L == l) {                                                                             \
         *cls = kBatchRealBase + idx;                                                          \
@@ -102,6 +152,21 @@ cudaError_t launch_sweep_batched(const PackedStep& ps, const RealStep& rs, const
                                  size_t smem, cudaStream_t st)
 {
     sweep_batch_kernel<<<blocks, kBatchThreads, smem, st>>>(ps, rs, insts, items, n_items, mult, counter);
+    return cudaGetLastError();
+}
+
+cudaError_t batch_table_occupancy(size_t smem, int* blocks_per_sm)
+{
+    cudaError_t e = cudaFuncSetAttribute(sweep_batch_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, sweep_batch_table_kernel, kTabThreads, smem);
+}
+
+cudaError_t launch_sweep_batched_table(const RealStep& rs, const BatchSweepInst* insts, const int2* items,
+                                       int n_items, int chunk, int* counter, int blocks, size_t smem, cudaStream_t st)
+{
+    sweep_batch_table_kernel<<<blocks, kTabThreads, smem, st>>>(rs, insts, items, n_items, chunk, counter);
     return cudaGetLastError();
 }
 

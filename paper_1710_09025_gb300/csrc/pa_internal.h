@@ -97,6 +97,7 @@ struct RealInst {
     const int* Rdev;         // population in device memory (or null: R); R then sizes the grid
     int R, NP;
     uint32_t c3;             // Philox counter word 3 of the WORD stream
+    int field;               // some h is not zero
 };
 struct RealSweepArgs {
     RealStep s;
@@ -105,6 +106,9 @@ struct RealSweepArgs {
 cudaError_t launch_sweep_real(int D, int L, const RealSweepArgs& a, int warps, int grid,
                               cudaStream_t st);
 bool real_supported(int D, int L);
+// whether the sweeps of this lattice run on threshold tables (else they
+// evaluate the field per attempt and use the guard band below)
+bool real_uses_table(int D, int L, bool field);
 // verifies the acceptance guard band for every positive finite float
 // (violations: count of x where it fails; max_rel_dev: largest |g/e - 1| for
 // 0 < x <= 87); synchronises st
@@ -118,17 +122,24 @@ cudaError_t launch_overlap_i8(const int8_t* A, const int8_t* B, int N, int NP, i
 
 // ---------------- batched sweep ----------------
 constexpr int kBatchRealBase = 100;   // class ids >= this are real-coupling tiles
+constexpr int kBatchTableBase = 200;  // class ids >= this are threshold-table chunks (their own launch)
+constexpr int kBatchTableGroups = 64; // most and fewest replica groups (of four) per chunk
+constexpr int kBatchTableLeast = 8;
 struct BatchSweepInst {
     int cls;                 // packed: 2 * lattice index (+1 for the doubled groups per block)
     int pad;
     PackedInst pk;
     RealInst re;
 };
-bool batch_class(int D, int L, int kind, int mult, int G, int R, int* cls, int* tiles, size_t* smem);
+bool batch_class(int D, int L, int kind, bool field, int mult, int chunk, int G, int R, int* cls, int* tiles,
+                 size_t* smem);
 cudaError_t batch_sweep_occupancy(size_t smem, int* blocks_per_sm);
 cudaError_t launch_sweep_batched(const PackedStep& ps, const RealStep& rs, const BatchSweepInst* insts,
                                  const int2* items, int n_items, int mult, int* counter, int blocks,
                                  size_t smem, cudaStream_t st);
+cudaError_t batch_table_occupancy(size_t smem, int* blocks_per_sm);
+cudaError_t launch_sweep_batched_table(const RealStep& rs, const BatchSweepInst* insts, const int2* items,
+                                       int n_items, int chunk, int* counter, int blocks, size_t smem, cudaStream_t st);
 
 // ---------------- isoenergetic cluster moves (Sec. II.C) ----------------
 struct IcmArgs {

@@ -15,6 +15,7 @@
 //
 // Energies are exact: E * 2^96 is an integer for FP32 couplings of magnitude
 // >= 2^-73, accumulated in int128, so the sum does not depend on order.
+#include "pa_real_table.cuh"
 #include "pa_sweep_tiles.cuh"
 
 #include <cstring>
@@ -145,14 +146,30 @@ bool real_supported(int D, int L)
     return false;
 }
 
+bool real_uses_table(int D, int L, bool field)
+{
+#define X(d, l) if (D == d && L == l) return field ? TabShape<d, l, true>::FITS : TabShape<d, l, false>::FITS;
+    PA_REAL_CASES(X)
+#undef X
+    return false;
+}
+
+// The threshold tables serve every lattice whose table fits in shared memory
+// (a block of 512 threads, one lookup per attempt); the rest (3D L = 12, and
+// 3D L = 10 with a field) evaluates the field and the guard band per attempt.
 cudaError_t launch_sweep_real(int D, int L, const RealSweepArgs& a, int warps, int grid,
                               cudaStream_t st)
 {
+    bool handled = false;
+    const cudaError_t e = a.i.field ? launch_sweep_real_table_field(D, L, a, st, &handled)
+                                    : launch_sweep_real_table_plain(D, L, a, st, &handled);
+    if (handled) return e;
 #define X(d, l)                                                                \
-    if (D == d && L == l) {                                                    \
-        if (warps == 4) return launch_real_one<d, l, 4>(a, grid, st);          \
-        return launch_real_one<d, l, 8>(a, grid, st);                          \
-    }
+    if constexpr (!TabShape<d, l, true>::FITS || !TabShape<d, l, false>::FITS) \
+        if (D == d && L == l) {                                                \
+            if (warps == 4) return launch_real_one<d, l, 4>(a, grid, st);      \
+            return launch_real_one<d, l, 8>(a, grid, st);                      \
+        }
     PA_REAL_CASES(X)
 #undef X
     return cudaErrorInvalidValue;
