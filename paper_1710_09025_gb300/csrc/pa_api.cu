@@ -41,7 +41,8 @@ struct pa_ctx {
     int icm;                    // isoenergetic cluster moves and their beta window
     double icm_lo, icm_hi;
     int* icm_err;               // device flag: a bounded union-find loop gave up
-    double* wtab;               // +-J: resampling weight per energy level
+    double *runP, *runq;        // resampling: run table
+    int32_t* bcount;            // resampling: copies per scan block
     int* sync;                  // block counters of the merged launches (zeroed)
     int* Rdev;                  // [n_temps] populations in device memory
     std::vector<float> Jh, hh;  // flushed host copies
@@ -153,7 +154,7 @@ __global__ void acc0_kernel(StepAcc* acc, double betaF0, int R, int* Rdev)
 enum {
     W_J, W_H, W_JNEG, W_JFIX, W_HFIX, W_BETAS, W_S0, W_S1, W_E32, W_E128, W_PARENT, W_FAM0, W_FAM1,
     W_COUNTS, W_BLOCKSUM, W_W, W_P, W_LEV1, W_BMAX, W_UPPER, W_ACC, W_CJ, W_CH, W_TMP8, W_HIST, W_GBAR, W_DJ,
-    W_DH, W_OBSPART, W_RK, W_RDEV, W_ICMERR, W_WTAB, W_SYNC, W_LOGC,
+    W_DH, W_OBSPART, W_RK, W_RDEV, W_ICMERR, W_RUNP, W_RUNQ, W_BCOUNT, W_SYNC, W_LOGC,
     W_SH_UPPER, W_SH_T2G, W_SH_BMAX, W_SH_POUT, W_SH_FOUT, W_SH_STAGE, W_COUNT
 };
 
@@ -210,7 +211,9 @@ static Layout make_layout(int D, int L, int kind, int layout, int R, int n_temps
     sz[W_RDEV] = sizeof(int) * n_temps;
     sz[W_ICMERR] = sizeof(int);
     sz[W_SYNC] = sizeof(int) * 4;
-    sz[W_WTAB] = kind == PA_PM1 ? sizeof(double) * (size_t)(D * N / 2 + 1) : 0;
+    sz[W_RUNP] = sizeof(double) * (size_t)pa::rs_leaves(R);
+    sz[W_RUNQ] = sizeof(double) * (size_t)pa::rs_leaves(R);
+    sz[W_BCOUNT] = sizeof(int32_t) * (size_t)pa::rs_bcount_size(R);
     if (shard_total > 0) {
         sz[W_SH_UPPER] = sizeof(double) * (size_t)pa::rs_upper_size(shard_total);
         sz[W_SH_T2G] = sizeof(double) * (size_t)pa::rs_wblocks(shard_total);
@@ -479,7 +482,7 @@ static int create_impl(pa_ctx** out, int D, int L, int kind, const float* J, con
     c->sh_upper = (double*)at(W_SH_UPPER); c->sh_t2g = (double*)at(W_SH_T2G); c->sh_bmax = (double*)at(W_SH_BMAX);
     c->sh_pout = (int32_t*)at(W_SH_POUT); c->sh_fout = (int32_t*)at(W_SH_FOUT);
     c->sh_stage = (uint64_t*)at(W_SH_STAGE);
-    c->wtab = kind == PA_PM1 ? (double*)at(W_WTAB) : nullptr;
+    c->runP = (double*)at(W_RUNP); c->runq = (double*)at(W_RUNQ); c->bcount = (int32_t*)at(W_BCOUNT);
 
     // couplings: sign masks (+-J), fixed-point copies (real)
     std::vector<uint8_t> jn(N, 0);
@@ -671,7 +674,7 @@ static void plan_step(pa_ctx* c, StepPlan* pl)
         ra.fam_in = c->fam[c->famcur]; ra.fam_out = c->fam[c->famcur ^ 1];
         ra.dbeta = c->betas[k] - c->betas[k - 1];
         ra.log_R = std::log((double)Rprev); ra.betaF0 = c->betaF0; ra.k = k;
-        ra.wtab = c->wtab; ra.wtab_n = c->wtab ? c->D * c->N / 2 + 1 : 0;  // E - E_min <= 2 D N
+        ra.runP = c->runP; ra.runq = c->runq; ra.bcount = c->bcount;
         ra.sync = c->sync;
         ra.key0 = k0; ra.key1 = k1; ra.c3 = pa::counter3(pa::STREAM_RES, c->tag, c->inst);
         c->famcur ^= 1;
@@ -820,7 +823,7 @@ static int enqueue_step(pa_ctx* c)
     if (k > 0) {
         ev = phase_begin(c, PA_PHASE_RESAMPLE);
         PA_CK(c, pa::launch_resample(pl.rs, c->st));
-        c->launches += pl.rs.wtab ? 6 : 5;
+        c->launches += pa::resample_launches(pl.rs);
         phase_end(c, PA_PHASE_RESAMPLE, ev);
     }
     if (pl.gather) {
@@ -1278,7 +1281,6 @@ static void shard_args(pa_ctx* c, pa::ResampleArgs* ra)
     ra->parent = c->sh_pout; ra->fam_in = c->fam[c->famcur]; ra->fam_out = c->sh_fout;
     ra->dbeta = c->betas[k] - c->betas[k - 1];
     ra->log_R = std::log((double)c->shard_total); ra->betaF0 = c->betaF0; ra->k = k;
-    ra->wtab = c->wtab; ra->wtab_n = c->D * c->N / 2 + 1;
     ra->key0 = (uint32_t)c->seed; ra->key1 = (uint32_t)(c->seed >> 32);
     ra->c3 = pa::counter3(pa::STREAM_RES, c->tag, c->inst);
 }
@@ -1310,7 +1312,7 @@ extern "C" int pa_shard_weights(pa_ctx* c, int64_t emin_global, double* host_blo
     PA_CK(c, cudaMemcpyAsync(host_block_totals, c->upper, sizeof(double) * pa::rs_wblocks(c->R),
                              cudaMemcpyDeviceToHost, c->st));
     PA_CK(c, cudaStreamSynchronize(c->st));
-    c->launches += 2;
+    c->launches += 1;
     return PA_OK;
 }
 
@@ -1671,15 +1673,11 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
             plan_step(c, &pl);
             const size_t at = (size_t)k * n_inst + i;
             rs[at] = pl.rs;
-            rs[at].wtab = nullptr;  // the batched resampling computes every weight
-            rs[at].wtab_n = 0;
-            rs[at].sync = nullptr;  // and launches every stage
             std::memset(&sw[at], 0, sizeof sw[at]);
             sw[at].cls = cls;
             sw[at].pk = pl.pk.i;
             sw[at].re = pl.re.i;
             ob[at] = pl.ob;
-            ob[at].sync = nullptr;
             b->after_cur[at] = pl.cur;
             b->after_fam[at] = pl.famcur;
         }
@@ -1849,7 +1847,7 @@ static int batch_enqueue(pa_batch* b, bool allow_tune)
         }
     } else {
         PB_CK(b, pa::launch_resample_batched(b->d_rs + (size_t)k * b->n_inst, b->n_inst, b->maxR, b->st));
-        b->launches += 8;
+        b->launches += 4;
     }
     if (!b->tuned && allow_tune && k >= 1) {
         int rc = batch_tune(b, k);
@@ -1882,7 +1880,7 @@ static int batch_enqueue(pa_batch* b, bool allow_tune)
         PB_CK(b, cudaStreamWaitEvent(b->st, b->ev_join, 0));
     }
     PB_CK(b, pa::launch_observe_batched(b->d_ob + (size_t)k * b->n_inst, b->n_inst, b->maxR, b->st));
-    b->launches += 2;
+    b->launches += 1;
     for (int i = 0; i < b->n_inst; ++i) {
         pa_ctx* c = b->ctx[i];
         c->k_next = k + 1;

@@ -170,15 +170,14 @@ struct ResampleArgs {
     const StepAcc* prev;         // acc[k-1]: E_min, sum_lnQ
     StepAcc* cur;                // acc[k]: lnQ, sum_lnQ, betaF, S
     double* w;                   // [R] weights
-    const double* wtab;          // +-J: weight per level (E - E_min) / 4, or null
-    int wtab_n;                  // levels in wtab
-    // two zeroed block counters: with them the last block of the weights
-    // launch completes the prefix (upper levels, run offsets, running maximum,
-    // S, ln Q) and the last block of the block-sum launch scans the block sums
-    // (no separate launches); null: separate launches
+    // zeroed block counters: the last block of the weights launch completes
+    // the prefix (sync[0]), that of the run table the running maximum (sync[3])
     int* sync;
-    double* P;                   // [R] sums inside runs of 32, then the cumulative weights
-                                 // up to the running maximum over earlier weights blocks
+    double* P;                   // [R] sums inside runs of 32 (a shard: then the cumulative weights
+                                 // up to the running maximum over earlier weights blocks)
+    double* runP;                // [rs_leaves(R)] run totals, then the largest cumulative weight up to
+                                 // the run's end inside its weights block
+    double* runq;                // [rs_leaves(R)] sum before each run
     double* lev1;                // [rs_leaves(R)] level-1 sums inside runs of 32 runs, then
                                  // the inclusive prefix of the run totals
     double* bmax;                // [2 rs_wblocks(R)] largest prefix sum of each weights block,
@@ -193,7 +192,9 @@ struct ResampleArgs {
     int gR, gb0;
     const double* t2g;
     int32_t* counts;             // [R] copy numbers (zero on entry, zeroed again on exit)
-    int32_t* blocksum;           // [nblocks] scratch for the count scan
+    int32_t* bcount;             // [rs_scan_blocks] copies per scan block
+    int32_t* blocksum;           // a shard: scratch for the count scan
+    double* lnQ_out;             // ln Q once more (or null)
     int32_t* parent;             // [R] out
     const int32_t* fam_in;       // [R]
     int32_t* fam_out;            // [R]
@@ -218,8 +219,20 @@ __host__ __device__ constexpr inline int rs_upper_size(int R)
         n = (n + kFan - 1) / kFan;
     }
 }
-constexpr int kScanBlock = 4096; // elements per block of the copy-number scan
+constexpr int kScanBlock = 4096; // elements per block of a shard's copy-number scan
+// replicas per block of the placement: small ones while that fills few SMs
+// (R = 10^5: 98 blocks instead of 25)
+constexpr int kSmallScanR = 131072;
+__host__ __device__ constexpr inline int rs_scan_size(int R) { return R <= kSmallScanR ? 1024 : 4096; }
+__host__ __device__ constexpr inline int rs_scan_blocks(int R) { return (R + rs_scan_size(R) - 1) / rs_scan_size(R); }
+// entries of bcount that serve every population up to R
+__host__ __device__ constexpr inline int rs_bcount_size(int R)
+{
+    const int s = rs_scan_blocks(R < kSmallScanR ? R : kSmallScanR), n = rs_scan_blocks(R);
+    return n > s ? n : s;
+}
 cudaError_t launch_resample(const ResampleArgs& a, cudaStream_t st);
+int resample_launches(const ResampleArgs& a);  // kernels that launch_resample enqueues
 // one phase (0..3) of a shard's resampling (a.gR > 0, a.sync null)
 cudaError_t launch_resample_shard(const ResampleArgs& a, int phase, cudaStream_t st);
 // all instances of a batch at once: tab[i] describes instance i (device memory)
@@ -250,7 +263,7 @@ struct ObsArgs {
     ObsPartial* part;            // [kObsBlocks] scratch
     const double* logc;          // [kLogC] log(c) for the family entropy (or null)
     StepAcc* cur;
-    int* sync;                   // zeroed block counter: the last block combines (or null)
+    int* sync;                   // zeroed block counter: the last block combines
 };
 // family sizes below kLogC take log(c) from a table that the context fills
 // once with the same device log; larger ones evaluate it

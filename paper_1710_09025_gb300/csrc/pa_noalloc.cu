@@ -26,20 +26,21 @@ namespace {
 constexpr int kMaxR = PA_STATIC_MAX_R;
 constexpr int kMaxLeaves = (kMaxR + pa::kFan - 1) / pa::kFan;
 constexpr int kMaxUpper = 2 * ((kMaxR + pa::kWBlock - 1) / pa::kWBlock) + 64;  // levels >= 2
-constexpr int kMaxScanBlocks = (kMaxR + pa::kScanBlock - 1) / pa::kScanBlock;
 
 // carve-up of the scratch array (byte offsets, each 256-byte aligned)
 constexpr size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
-constexpr size_t kOffW = 0;
-constexpr size_t kOffP = kOffW + al(sizeof(double) * kMaxR);
+constexpr size_t kOffP = 0;
 constexpr size_t kOffCounts = kOffP + al(sizeof(double) * kMaxR);
 constexpr size_t kOffFamIn = kOffCounts + al(sizeof(int32_t) * kMaxR);
 constexpr size_t kOffFamOut = kOffFamIn + al(sizeof(int32_t) * kMaxR);
 constexpr size_t kOffLev1 = kOffFamOut + al(sizeof(int32_t) * kMaxR);
 constexpr size_t kOffBmax = kOffLev1 + al(sizeof(double) * kMaxLeaves);
 constexpr size_t kOffUpper = kOffBmax + al(sizeof(double) * 2 * ((kMaxR + pa::kWBlock - 1) / pa::kWBlock));
-constexpr size_t kOffBlock = kOffUpper + al(sizeof(double) * kMaxUpper);
-constexpr size_t kOffAcc = kOffBlock + al(sizeof(int32_t) * (kMaxScanBlocks + 1));
+constexpr size_t kOffRunP = kOffUpper + al(sizeof(double) * kMaxUpper);
+constexpr size_t kOffRunQ = kOffRunP + al(sizeof(double) * kMaxLeaves);
+constexpr size_t kOffCount = kOffRunQ + al(sizeof(double) * kMaxLeaves);
+constexpr size_t kOffSync = kOffCount + al(sizeof(int32_t) * pa::rs_bcount_size(kMaxR));
+constexpr size_t kOffAcc = kOffSync + al(sizeof(int) * 4);
 constexpr size_t kBytes = kOffAcc + al(2 * sizeof(pa::StepAcc));
 static_assert(kBytes <= PA_STATIC_SCRATCH_BYTES, "scratch layout exceeds the stated size");
 static_assert(pa::rs_upper_size(kMaxR) <= kMaxUpper, "upper prefix levels fit");
@@ -75,17 +76,14 @@ __global__ void __launch_bounds__(1024) static_prep_kernel(const int32_t* E, int
     if (threadIdx.x < 32) {
         int v = __reduce_min_sync(0xffffffffu, wmin[threadIdx.x]);
         if (threadIdx.x == 0) {
+            int* sync = reinterpret_cast<int*>(base + kOffSync);
+            for (int t = 0; t < 4; ++t) sync[t] = 0;
             acc[0] = pa::StepAcc{};
             acc[1] = pa::StepAcc{};
             acc[0].emin_lo = v;
             acc[0].emin_hi = v < 0 ? -1 : 0;
         }
     }
-}
-
-__global__ void static_lnq_kernel(const unsigned char* base, double* lnQ)
-{
-    *lnQ = reinterpret_cast<const pa::StepAcc*>(base + kOffAcc)[1].lnQ;
 }
 
 }  // namespace
@@ -141,13 +139,16 @@ extern "C" int pa_resample_static(const int32_t* d_E, int R, double beta_prev, d
     ra.E128 = nullptr;
     ra.prev = reinterpret_cast<const pa::StepAcc*>(base + kOffAcc);
     ra.cur = reinterpret_cast<pa::StepAcc*>(base + kOffAcc) + 1;
-    ra.w = reinterpret_cast<double*>(base + kOffW);
     ra.P = reinterpret_cast<double*>(base + kOffP);
     ra.lev1 = reinterpret_cast<double*>(base + kOffLev1);
     ra.bmax = reinterpret_cast<double*>(base + kOffBmax);
     ra.upper = reinterpret_cast<double*>(base + kOffUpper);
     ra.counts = reinterpret_cast<int32_t*>(base + kOffCounts);
-    ra.blocksum = reinterpret_cast<int32_t*>(base + kOffBlock);
+    ra.runP = reinterpret_cast<double*>(base + kOffRunP);
+    ra.runq = reinterpret_cast<double*>(base + kOffRunQ);
+    ra.bcount = reinterpret_cast<int32_t*>(base + kOffCount);
+    ra.sync = reinterpret_cast<int*>(base + kOffSync);
+    ra.lnQ_out = d_lnQ;
     ra.parent = d_parent;
     ra.fam_in = reinterpret_cast<const int32_t*>(base + kOffFamIn);
     ra.fam_out = reinterpret_cast<int32_t*>(base + kOffFamOut);
@@ -159,10 +160,6 @@ extern "C" int pa_resample_static(const int32_t* d_E, int R, double beta_prev, d
     ra.key1 = (uint32_t)(seed >> 32);
     ra.c3 = pa::counter3(pa::STREAM_RES, rng_tag, rng_instance);
     e = pa::launch_resample(ra, st);
-    if (e == cudaSuccess) {
-        static_lnq_kernel<<<1, 1, 0, st>>>(base, d_lnQ);
-        e = cudaGetLastError();
-    }
     if (e != cudaSuccess) {
         pa::set_global_error((std::string("pa_resample_static: ") + cudaGetErrorString(e)).c_str());
         return PA_ECUDA;

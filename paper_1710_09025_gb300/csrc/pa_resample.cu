@@ -33,17 +33,17 @@ __device__ __forceinline__ double e_minus_min_to_double(const ResampleArgs& a, i
     return __dmul_rn(i128_to_double(ll2_to_i128(a.E128[i]) - emin), 0x1p-96);
 }
 
-// true in the block that finishes last (every block calls it once); the
+// true in the block that finishes last (each of n_blocks calls it once); the
 // counter is reset for the next launch.  Writes before the call are visible
 // to the last block (fence before the count).
-__device__ __forceinline__ bool last_block(int* counter)
+__device__ __forceinline__ bool last_block(int* counter, int n_blocks)
 {
     __shared__ int s_last;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         const int done = atomicAdd(counter, 1);
-        s_last = done == (int)(gridDim.x * gridDim.y) - 1;
+        s_last = done == n_blocks - 1;
         if (s_last) *counter = 0;
     }
     __syncthreads();
@@ -51,106 +51,245 @@ __device__ __forceinline__ bool last_block(int* counter)
     return s_last;
 }
 
+constexpr int kWThreads = 256;
+
 // source population: in device memory for the nearest-integer scheme
 __device__ __forceinline__ int rs_src(const ResampleArgs& a) { return a.Rsrc ? *a.Rsrc : a.R; }
 
-// Weights and the two lowest levels of the prefix, one block of kWThreads
-// threads per kWBlock weights (small blocks, so that several blocks' FP64
-// chains overlap on an SM).  GB300 has little FP64 throughput, so every
-// addition of the specified order is executed once: lane c of warp 0 sums
-// run c (32 weights, staged in shared memory, loaded eight at a time) left
-// to right, then lane 0 sums the block's run totals left to right.
-constexpr int kWThreads = 256;
-__device__ __forceinline__ void rs_weights_body(const ResampleArgs& a, int b)
+// Weights and the two lowest levels of the prefix, one block of T threads per
+// kWBlock weights.  GB300 has little FP64 throughput (two operations a clock
+// and SM), so every operation of the specified order is executed once: thread c
+// of the first warp sums run c (32 weights, staged in shared memory) left to
+// right, then one thread sums the block's run totals left to right.  +-J
+// energies of a block span a few dozen to a few hundred levels, so the block
+// evaluates each level's weight once (spec_exp64 of the same argument) and looks
+// the weights up.
+//
+// Two shapes.  Populations of at most kFuseR: 1024 threads, one weight each, and
+// the last block to finish completes the prefix, the run search table and S
+// (rs_fused): with at most 128 blocks the launch is latency alone, and a second
+// and third launch cost more than one SM's work.  Larger ones: 256 threads, so
+// that several blocks' dependent FP64 chains overlap on an SM, and the run table
+// is its own launch (rs_runs_kernel).  R = 10^5, by ncu: level table + weights +
+// finalize 24 us -> 16 us, most of it 62-cycle FP64 additions in a chain.
+constexpr int kFuseR = 128 * kWBlock;
+template <int T>
+__device__ __forceinline__ void rs_levels_body(const ResampleArgs& a, int b, int R)
 {
+    constexpr int PER = kWBlock / T;
     __shared__ double s_w[kFan * (kFan + 1)];  // run c at [c (kFan + 1)], padded against bank conflicts
-    __shared__ double s_t[kFan];
-    const int R = rs_src(a);
+    __shared__ double s_t[kFan], s_l1[kFan];
+    __shared__ int s_lo[T / 32], s_hi[T / 32];
     const int i0 = b * kWBlock;
-    if (i0 >= R) return;  // block-uniform: past the source population
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = min(kWBlock, R - i0);
-    for (int t = tid; t < n; t += kWThreads) {
-        const int i = i0 + t;
-        double w;
-        const int lv = a.kind == 0 ? a.E32[i] - (int)a.prev->emin_lo : 0;
-        if (a.wtab && (lv & 3) == 0 && (lv >> 2) < a.wtab_n) {
-            w = a.wtab[lv >> 2];  // +-J: E - E_min is a multiple of 4, the weight a table entry
-        } else {
-            const double d = e_minus_min_to_double(a, i);
-            w = spec_exp64(-__dmul_rn(a.dbeta, d));
+    if (tid == 0 && a.bcount && b < rs_scan_blocks(R)) a.bcount[b] = 0;
+    if (a.kind == 0) {
+        const int emin = (int)a.prev->emin_lo;
+        int lv[PER], lo = 0x7fffffff, hi = -1;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int t = tid + j * T;
+            lv[j] = t < n ? a.E32[i0 + t] - emin : -1;
+            if (t < n) {
+                lo = min(lo, lv[j]);
+                hi = max(hi, (lv[j] & 3) ? 0x7ffffffe : lv[j]);  // not a level: no table
+            }
         }
-        a.w[i] = w;
-        s_w[(t / kFan) * (kFan + 1) + t % kFan] = w;
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (lane == 0) { s_lo[warp] = lo; s_hi[warp] = hi; }
+        __syncthreads();
+        lo = __reduce_min_sync(0xffffffffu, lane < T / 32 ? s_lo[lane] : 0x7fffffff);
+        hi = __reduce_max_sync(0xffffffffu, lane < T / 32 ? s_hi[lane] : -1);
+        // levels lo/4 .. hi/4 evaluated once each (staged in s_w, read before the weights replace them)
+        const int nlev = hi < 0x7ffffff0 && lo >= 0 ? (hi >> 2) - (lo >> 2) + 1 : kWBlock;
+        double w[PER];
+        if (nlev <= kWBlock / 2) {
+            for (int t = tid; t < nlev; t += T)
+                s_w[t] = spec_exp64(-__dmul_rn(a.dbeta, (double)(4 * ((lo >> 2) + t))));
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < PER; ++j) w[j] = lv[j] >= 0 ? s_w[(lv[j] >> 2) - (lo >> 2)] : 0.0;
+        } else {
+#pragma unroll
+            for (int j = 0; j < PER; ++j)
+                w[j] = tid + j * T < n ? spec_exp64(-__dmul_rn(a.dbeta, (double)lv[j])) : 0.0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int t = tid + j * T;
+            if (t < n) s_w[(t / kFan) * (kFan + 1) + t % kFan] = w[j];
+            if (t < n && a.scheme == 1) a.w[i0 + t] = w[j];
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int t = tid + j * T;
+            if (t >= n) continue;
+            const double w = spec_exp64(-__dmul_rn(a.dbeta, e_minus_min_to_double(a, i0 + t)));
+            if (a.scheme == 1) a.w[i0 + t] = w;
+            s_w[(t / kFan) * (kFan + 1) + t % kFan] = w;
+        }
     }
     __syncthreads();
     const int nruns = (n + kFan - 1) / kFan;
-    if (tid < nruns) {  // run tid, left to right
-        double* x = s_w + tid * (kFan + 1);
-        const int cnt = min(kFan, n - tid * kFan);
-        double acc = 0.0;
-        for (int j0 = 0; j0 < cnt; j0 += 8) {
-            double v[8];
+    if (warp == 0) {
+        double tot = 0.0;
+        if (lane < nruns) {  // run `lane`, left to right
+            double* x = s_w + lane * (kFan + 1);
+            const int cnt = min(kFan, n - lane * kFan);
+            double acc = 0.0;
+            for (int j0 = 0; j0 < cnt; j0 += 8) {
+                double v[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = j0 + j < cnt ? x[j0 + j] : 0.0;
+                for (int j = 0; j < 8; ++j) v[j] = j0 + j < cnt ? x[j0 + j] : 0.0;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (j0 + j < cnt) {
-                    acc = (j0 + j == 0) ? v[0] : __dadd_rn(acc, v[j]);
-                    x[j0 + j] = acc;
+                for (int j = 0; j < 8; ++j) {
+                    if (j0 + j < cnt) {
+                        acc = (j0 + j == 0) ? v[0] : __dadd_rn(acc, v[j]);
+                        x[j0 + j] = acc;
+                    }
                 }
             }
+            tot = acc;
+            s_t[lane] = acc;
         }
-        s_t[tid] = acc;
+        __syncwarp();
+        if (lane == 0) {  // the block's run totals, left to right
+            double acc = n > 0 ? s_t[0] : 0.0;
+            s_l1[0] = acc;
+            for (int c = 1; c < nruns; ++c) {
+                acc = __dadd_rn(acc, s_t[c]);
+                s_l1[c] = acc;
+            }
+            a.upper[b] = acc;
+        }
+        __syncwarp();
+        if (lane < nruns) {
+            a.lev1[b * kFan + lane] = s_l1[lane];
+            if (a.runP) a.runP[b * kFan + lane] = tot;
+        }
     }
     __syncthreads();
-    for (int t = tid; t < n; t += kWThreads) a.P[i0 + t] = s_w[(t / kFan) * (kFan + 1) + t % kFan];
-    if (tid == 0) {  // the block's run totals, left to right
-        double acc = s_t[0];
-        a.lev1[b * kFan] = acc;
-        for (int c = 1; c < nruns; ++c) {
-            acc = __dadd_rn(acc, s_t[c]);
-            a.lev1[b * kFan + c] = acc;
+    for (int t = tid; t < n; t += T) a.P[i0 + t] = s_w[(t / kFan) * (kFan + 1) + t % kFan];
+}
+
+// one weights block's run table, by one warp (lane = run c): q_c, the sum of
+// everything before the run (Q1_{c-1}), and the largest cumulative weight up to
+// the run's end inside the block; returns the block's largest.  Inside a run
+// q_c + l_i does not decrease, so the smallest i with P_i > x lies in the first
+// run whose entry here exceeds x: the cumulative weights themselves are never
+// written out.
+__device__ __forceinline__ long long dbits(double x);
+__device__ __forceinline__ long long rs_run_table(const ResampleArgs& a, int b, int R, const double* upper)
+{
+    const int lane = threadIdx.x & 31, c = b * kFan + lane;
+    double q = 0.0;
+    long long m = 0;  // bits of +0.0: weights are >= 0
+    const bool live = (long long)c * kFan < R;
+    if (live) {
+        const double tot = __ldcg(a.runP + c);
+        if (c > 0) {
+            const double l1 = __ldcg(a.lev1 + c - 1);
+            const int cb = (c - 1) / kFan;  // block of run c - 1
+            q = cb == 0 ? l1 : __dadd_rn(upper[cb - 1], l1);
         }
-        a.upper[b] = acc;
+        m = dbits(c == 0 ? tot : __dadd_rn(q, tot));
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long u = __shfl_up_sync(0xffffffffu, m, o);
+        if (lane >= o) m = max(m, u);
+    }
+    if (live) {
+        a.runq[c] = q;
+        a.runP[c] = __longlong_as_double(m);
+    }
+    return __shfl_sync(0xffffffffu, m, 31);
+}
+
+__device__ __forceinline__ void rs_top_levels(double* up, int nb);
+// the last weights block of a population of at most kFuseR: levels >= 2 of the
+// prefix, run table, running maximum over the blocks, S
+__device__ __forceinline__ void rs_fused(const ResampleArgs& a, int R)
+{
+    constexpr int kNb = kFuseR / kWBlock;
+    __shared__ double s_up[rs_upper_size(kFuseR)];
+    __shared__ long long s_bm[kNb];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nb = rs_wblocks(R);
+    for (int t = tid; t < nb; t += blockDim.x) s_up[t] = __ldcg(a.upper + t);
+    if (tid < kNb) s_bm[tid] = 0;
+    __syncthreads();
+    rs_top_levels(s_up, nb);
+    for (int b = warp; b < nb; b += blockDim.x / 32) {
+        const long long m = rs_run_table(a, b, R, s_up);
+        if (lane == 0) s_bm[b] = m;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        constexpr int PER = kNb / 32;
+        long long v[PER], m = 0;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) { m = max(m, s_bm[lane * PER + j]); v[j] = m; }
+        long long inc = m;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc = max(inc, u);
+        }
+        long long before = __shfl_up_sync(0xffffffffu, inc, 1);
+        if (lane == 0) before = 0;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int b = lane * PER + j;
+            if (b < nb) a.bmax[nb + b] = __longlong_as_double(j == 0 ? before : max(before, v[j - 1]));
+        }
+        if (lane == 31) a.cur->S = __longlong_as_double(inc);
     }
 }
 __device__ __forceinline__ void rs_top_body(const ResampleArgs& a);
-__global__ void __launch_bounds__(kWThreads) rs_weights_kernel(ResampleArgs a)
+// blocks of an instance that take part (block 0 always: it resets the copy
+// totals and S even of a population that died out)
+__device__ __forceinline__ int rs_live_blocks(int R) { return max(1, rs_wblocks(R)); }
+template <int T>
+__device__ __forceinline__ void rs_weights_launch(const ResampleArgs& a, int b)
 {
-    rs_weights_body(a, blockIdx.x);
-    if (a.sync && last_block(a.sync)) rs_top_body(a);  // levels >= 2 of the prefix
+    const int R = rs_src(a), live = rs_live_blocks(R);
+    if (b >= live) return;  // block-uniform: past the source population
+    rs_levels_body<T>(a, b, R);
+    if (!last_block(a.sync, live)) return;
+    if (T == kWBlock) rs_fused(a, R);
+    else rs_top_body(a);  // levels >= 2 of the prefix
 }
+__global__ void __launch_bounds__(kWBlock) rs_weights_fused_kernel(ResampleArgs a) { rs_weights_launch<kWBlock>(a, blockIdx.x); }
+__global__ void __launch_bounds__(kWThreads) rs_weights_kernel(ResampleArgs a) { rs_weights_launch<kWThreads>(a, blockIdx.x); }
 __global__ void __launch_bounds__(kWThreads) rs_weights_batched(const ResampleArgs* tab)
 {
-    const ResampleArgs& a = tab[blockIdx.y];
-    rs_weights_body(a, blockIdx.x);
+    rs_weights_launch<kWThreads>(tab[blockIdx.y], blockIdx.x);
 }
-
-// +-J: all energies are congruent modulo 4 (Delta E of a flip is 4D - 4n),
-// so E - E_min takes the values 4l, l < wtab_n; the weight of level l,
-// spec_exp64(-(dbeta * 4l)), is the same arithmetic as for a replica
-__global__ void rs_table_kernel(ResampleArgs a)
+// a shard: the levels >= 2 need every shard's block totals
+__global__ void __launch_bounds__(kWThreads) rs_weights_shard_kernel(ResampleArgs a)
 {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l < a.wtab_n) const_cast<double*>(a.wtab)[l] = spec_exp64(-__dmul_rn(a.dbeta, (double)(4 * l)));
+    rs_levels_body<kWThreads>(a, blockIdx.x, a.R);
 }
 
-// Levels >= 2 of the prefix, by one block of kWBlock threads after every
-// weights block is done: bottom-up sums inside runs of the block totals (each
-// thread loads its run, then adds in order), then top-down Q_{c-1} + l_j.
-__device__ __forceinline__ void rs_top_body(const ResampleArgs& a)
+// Levels >= 2 of the prefix, by one block: bottom-up sums inside runs of the nb
+// block totals at up (each thread loads its run, then adds in order), then
+// top-down Q_{c-1} + l_j; up[0 .. nb) ends as the inclusive prefix.
+__device__ __forceinline__ void rs_top_levels(double* up, int nb)
 {
     constexpr int kMaxLev = 8;  // kFan^(kMaxLev+1) > 2^31 weights
     const int tid = threadIdx.x, nt = blockDim.x;
-    const int R = a.gR ? a.gR : rs_src(a);  // a shard sums the global block totals
     int base[kMaxLev], len[kMaxLev], nl = 0;
-    int n = rs_wblocks(R), off = 0;
+    int n = nb, off = 0;
     for (;;) {
         base[nl] = off; len[nl] = n; ++nl;
         const int nc = n <= kFan ? 1 : (n + kFan - 1) / kFan;
         for (int c = tid; c < nc; c += nt) {
-            double* x = a.upper + off + c * kFan;
+            double* x = up + off + c * kFan;
             const int cnt = min(kFan, n - c * kFan);
             double acc = 0.0;
             for (int j0 = 0; j0 < cnt; j0 += 8) {  // eight independent loads, then the additions
@@ -166,7 +305,7 @@ __device__ __forceinline__ void rs_top_body(const ResampleArgs& a)
                 for (int j = 0; j < 8; ++j)
                     if (j0 + j < cnt) x[j0 + j] = v[j];
             }
-            if (n > kFan) a.upper[off + n + c] = acc;
+            if (n > kFan) up[off + n + c] = acc;
         }
         __syncthreads();
         if (n <= kFan) break;  // one run left: its sums are the prefix of this level
@@ -174,25 +313,24 @@ __device__ __forceinline__ void rs_top_body(const ResampleArgs& a)
         n = nc;
     }
     for (int v = nl - 2; v >= 0; --v) {
-        double* x = a.upper + base[v];
-        const double* q = a.upper + base[v + 1];
+        double* x = up + base[v];
+        const double* q = up + base[v + 1];
         for (int j = kFan + tid; j < len[v]; j += nt) x[j] = __dadd_rn(q[j / kFan - 1], x[j]);
         __syncthreads();
     }
 }
-__global__ void __launch_bounds__(kWBlock) rs_top_kernel(ResampleArgs a) { rs_top_body(a); }
-// one block per instance
-__global__ void __launch_bounds__(kWBlock) rs_top_batched(const ResampleArgs* tab, int n_inst)
+__device__ __forceinline__ void rs_top_body(const ResampleArgs& a)
 {
-    if ((int)blockIdx.x < n_inst) rs_top_body(tab[blockIdx.x]);
+    rs_top_levels(a.upper, rs_wblocks(a.gR ? a.gR : rs_src(a)));  // a shard sums the global block totals
 }
+__global__ void __launch_bounds__(kWBlock) rs_top_kernel(ResampleArgs a) { rs_top_body(a); }
 
 // Non-negative doubles compare as their bit patterns do (as signed 64-bit
 // integers): maxima and the draw search use the integer compare, which is
 // exact and leaves GB300's scarce FP64 units to the specified additions.
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
 
-// Level 0 and the running maximum inside one weights block: weight i of run
+// (shards) Level 0 and the running maximum inside one weights block: weight i of run
 // c gets Q1_{c-1} + l_i (Q1_{c-1} = Q2_{b'-1} + l1_{c-1} with b' the block of
 // run c - 1, the level-1 sums alone in block 0), then P_i = the largest of
 // these up to i within the block; bmax[b] = the block's largest.
@@ -255,9 +393,9 @@ __device__ __forceinline__ void rs_finalize_body(const ResampleArgs& a, int b)
     }
 }
 // running maximum over the weights blocks (bmax[nb + b] = the largest
-// cumulative weight before block b), S = the largest cumulative weight, ln Q
-// and the running free energy; one block, as many block maxima per pass as it
-// has threads (integer maxima of the bit patterns)
+// cumulative weight before block b) and S, the largest cumulative weight; one
+// block, as many block maxima per pass as it has threads (integer maxima of the
+// bit patterns)
 __device__ __forceinline__ void rs_blockmax_body(const ResampleArgs& a)
 {
     __shared__ long long s_w[32];
@@ -287,8 +425,12 @@ __device__ __forceinline__ void rs_blockmax_body(const ResampleArgs& a)
         if (tid == nt - 1) s_carry = max(before, m);
         __syncthreads();
     }
-    if (tid != 0) return;
-    const double S = __longlong_as_double(s_carry);
+    if (tid == 0) a.cur->S = __longlong_as_double(s_carry);
+}
+// ln Q and the running free energy, by one thread, once S is there
+__device__ __forceinline__ void rs_lnq(const ResampleArgs& a)
+{
+    const double S = a.cur->S;
     double emin_d;
     if (a.kind == 0) {
         emin_d = (double)(int)a.prev->emin_lo;
@@ -296,96 +438,124 @@ __device__ __forceinline__ void rs_blockmax_body(const ResampleArgs& a)
         __int128 emin = ((__int128)a.prev->emin_hi << 64) | (unsigned long long)a.prev->emin_lo;
         emin_d = __dmul_rn(i128_to_double(emin), 0x1p-96);
     }
-    const double log_R = a.Rsrc ? log((double)R) : a.log_R;
+    const double log_R = a.Rsrc ? log((double)rs_src(a)) : a.log_R;
     const double lnQ = __dsub_rn(__dadd_rn(-__dmul_rn(a.dbeta, emin_d), log(S)), log_R);
     const double sum = __dadd_rn(a.prev->sum_lnQ, lnQ);
     a.cur->lnQ = lnQ;
     a.cur->sum_lnQ = sum;
     a.cur->betaF = __dsub_rn(a.betaF0, sum);
-    a.cur->S = S;
+    if (a.lnQ_out) *a.lnQ_out = lnQ;
 }
-__global__ void __launch_bounds__(kWThreads) rs_finalize_kernel(ResampleArgs a)
+__global__ void __launch_bounds__(kWThreads) rs_finalize_shard_kernel(ResampleArgs a) { rs_finalize_body(a, blockIdx.x); }
+__global__ void __launch_bounds__(kWBlock) rs_blockmax_shard_kernel(ResampleArgs a)
 {
-    rs_finalize_body(a, blockIdx.x);
-    if (a.sync && last_block(a.sync + 3)) rs_blockmax_body(a);
-}
-__global__ void __launch_bounds__(kWThreads) rs_finalize_batched(const ResampleArgs* tab)
-{
-    rs_finalize_body(tab[blockIdx.y], blockIdx.x);
-}
-__global__ void __launch_bounds__(kWBlock) rs_blockmax_kernel(ResampleArgs a) { rs_blockmax_body(a); }
-// one block per instance
-__global__ void __launch_bounds__(kWBlock) rs_blockmax_batched(const ResampleArgs* tab, int n_inst)
-{
-    if ((int)blockIdx.x < n_inst) rs_blockmax_body(tab[blockIdx.x]);
+    rs_blockmax_body(a);
+    __syncthreads();
+    if (threadIdx.x == 0) rs_lnq(a);
 }
 
-// Multinomial draws.  P is non-decreasing, so the smallest i with x < P_i
-// lies in the first segment (of s consecutive weights, whole weights blocks)
-// whose last P exceeds x: each block stages the segment ends in shared memory,
-// finds the segment there and bisects only inside it in global memory.  P_i
-// is the stored block-local value raised to the largest value before its
-// weights block.
+// the run table of a population above kFuseR: one warp per weights block, the
+// last block takes the running maximum over the weights blocks and S
+constexpr int kRunWarps = 8;
+__device__ __forceinline__ void rs_runs_launch(const ResampleArgs& a, int blk)
+{
+    const int R = rs_src(a), nb = rs_wblocks(R), live = max(1, (nb + kRunWarps - 1) / kRunWarps);
+    if (blk >= live) return;
+    const int b = blk * kRunWarps + (threadIdx.x >> 5);
+    if (b < nb) {
+        const long long m = rs_run_table(a, b, R, a.upper);
+        if ((threadIdx.x & 31) == 0) a.bmax[b] = __longlong_as_double(m);
+    }
+    if (last_block(a.sync + 3, live)) rs_blockmax_body(a);
+}
+__global__ void __launch_bounds__(32 * kRunWarps) rs_runs_kernel(ResampleArgs a) { rs_runs_launch(a, blockIdx.x); }
+__global__ void __launch_bounds__(32 * kRunWarps) rs_runs_batched(const ResampleArgs* tab)
+{
+    rs_runs_launch(tab[blockIdx.y], blockIdx.x);
+}
+
+// Multinomial draws: the smallest i with x < P_i.  Each block stages the ends of
+// the segments of P (whole weights blocks) in shared memory and finds a draw's
+// segment there; the block's run table gives the run and the sums inside the run
+// the index, four ways at a time (three independent loads a round, three rounds
+// each, instead of ten dependent loads).  Copies are counted per replica and,
+// through shared memory, per scan block, so that the placement needs no pass
+// over the counts first.
 constexpr int kDrawThreads = 512;
+constexpr int kDrawSmall = 256;  // populations of at most kFuseR: more, smaller blocks
 constexpr int kMaxSeg = 2048;
+constexpr int kMaxHist = 1024;   // scan blocks counted in shared memory
 __device__ __forceinline__ int rs_seg_blocks(int nb)
 {
     int s = 1;
     while ((nb + s - 1) / s > kMaxSeg) s *= 2;
     return s;
 }
-__device__ __forceinline__ long long rs_P(const ResampleArgs& a, int nb, int i)
+// the first index of 32 where pred holds (it holds somewhere, and from there on)
+template <class Pred>
+__device__ __forceinline__ int first_of_32(Pred pred)
 {
-    return max(dbits(a.bmax[nb + i / kWBlock]), dbits(a.P[i]));
+    const bool p7 = pred(7), p15 = pred(15), p23 = pred(23);
+    int lo = p7 ? 0 : p15 ? 8 : p23 ? 16 : 24;
+    const bool q1 = pred(lo + 1), q3 = pred(lo + 3), q5 = pred(lo + 5);
+    lo += q1 ? 0 : q3 ? 2 : q5 ? 4 : 6;
+    return pred(lo) ? lo : lo + 1;
 }
-__device__ __forceinline__ void rs_draws_body(const ResampleArgs& a, int q)
+__device__ __forceinline__ void rs_draws_body(const ResampleArgs& a, int q0, int per)
 {
     __shared__ long long s_end[kMaxSeg];
-    const int R = a.R;
-    const int nb = rs_wblocks(R);
-    const int sb = rs_seg_blocks(nb), seg = sb * kWBlock, nseg = (nb + sb - 1) / sb;
+    __shared__ int s_hist[kMaxHist];
+    const int R = a.R, tid = threadIdx.x, nt = blockDim.x;
+    const int nb = rs_wblocks(R), leaves = rs_leaves(R);
+    const int sb = rs_seg_blocks(nb), nseg = (nb + sb - 1) / sb;
+    const int ns = rs_scan_blocks(R), sbits = rs_scan_size(R);
+    const bool hist = ns <= kMaxHist;
     const double S = a.cur->S;
-    for (int k = threadIdx.x; k < nseg; k += blockDim.x) {
-        const int lb = min(nb - 1, k * sb + sb - 1);  // last weights block of segment k
-        // its largest P: the largest before the next block, or S for the last block
-        s_end[k] = lb + 1 < nb ? dbits(a.bmax[nb + lb + 1]) : dbits(S);
-    }
+    // largest P up to the end of block b: the largest before block b + 1, or S
+    auto block_end = [&](int b) { return b + 1 < nb ? dbits(a.bmax[nb + b + 1]) : dbits(S); };
+    for (int k = tid; k < nseg; k += nt) s_end[k] = block_end(min(nb - 1, k * sb + sb - 1));
+    if (hist)
+        for (int k = tid; k < ns; k += nt) s_hist[k] = 0;
     __syncthreads();
-    if (q >= a.Rn) return;
-    const u32x4 o = philox((uint32_t)q, (uint32_t)a.k, 0u, a.c3, a.key0, a.key1);
-    const long long x = dbits(__dmul_rn(uniform53(o.x, o.y), S));  // x >= 0
-    int lo = 0, hi = nseg;  // first segment whose end exceeds x
-    while (lo < hi) {
-        const int mid = lo + ((hi - lo) >> 1);
-        if (x < s_end[mid]) hi = mid; else lo = mid + 1;
-    }
-    if (lo < nseg) {
-        const int k = lo;
-        lo = k * seg;
-        hi = min(R - 1, k * seg + seg - 1);  // x < P[hi]
-        if (sb == 1) {
-            // one weights block: x is at least the largest P before it, so
-            // x < max(that, stored P_i) reduces to x < stored P_i
-            while (lo < hi) {
-                const int mid = lo + ((hi - lo) >> 1);
-                if (x < dbits(a.P[mid])) hi = mid; else lo = mid + 1;
-            }
-        } else {
-            while (lo < hi) {
-                const int mid = lo + ((hi - lo) >> 1);
-                if (x < rs_P(a, nb, mid)) hi = mid; else lo = mid + 1;
-            }
-        }
-    } else {
-        // x == S after rounding: the smallest i with P_i >= x
-        lo = 0; hi = R;
+    for (int d = 0; d < per; ++d) {
+        const int q = q0 + d * nt + tid;
+        if (q >= a.Rn) break;
+        const u32x4 o = philox((uint32_t)q, (uint32_t)a.k, 0u, a.c3, a.key0, a.key1);
+        const long long x = dbits(__dmul_rn(uniform53(o.x, o.y), S));  // x >= 0
+        int lo = 0, hi = nseg;  // first segment whose end exceeds x
         while (lo < hi) {
             const int mid = lo + ((hi - lo) >> 1);
-            if (rs_P(a, nb, mid) >= x) hi = mid; else lo = mid + 1;
+            if (x < s_end[mid]) hi = mid; else lo = mid + 1;
         }
-        if (lo >= R) lo = R - 1;  // unreachable: x = u S <= S = P[R-1]
+        const bool strict = lo < nseg;  // some P exceeds x; else x == S after rounding: the first P >= x
+        int b0 = strict ? lo * sb : 0, b1 = strict ? min(nb - 1, lo * sb + sb - 1) : nb - 1;
+        while (b0 < b1) {
+            const int mid = b0 + ((b1 - b0) >> 1);
+            const long long e = block_end(mid);
+            if (strict ? x < e : e >= x) b1 = mid; else b0 = mid + 1;
+        }
+        // the largest P before the block does not pass the test, so neither it
+        // nor the runs before the first that does matter
+        const int c = b0 * kFan + first_of_32([&](int t) {
+            if (b0 * kFan + t >= leaves) return true;
+            const long long p = dbits(a.runP[b0 * kFan + t]);
+            return strict ? x < p : p >= x;
+        });
+        const double qc = a.runq[min(c, leaves - 1)];
+        const int i = c * kFan + first_of_32([&](int t) {
+            if (c * kFan + t >= R) return true;
+            const long long p = dbits(__dadd_rn(qc, a.P[c * kFan + t]));
+            return strict ? x < p : p >= x;
+        });
+        const int w = min(i, R - 1);
+        atomicAdd(&a.counts[w], 1);
+        if (hist) atomicAdd(&s_hist[w / sbits], 1);
+        else atomicAdd(&a.bcount[w / sbits], 1);
     }
-    atomicAdd(&a.counts[lo], 1);
+    if (!hist) return;  // block-uniform
+    __syncthreads();
+    for (int k = tid; k < ns; k += nt)
+        if (s_hist[k]) atomicAdd(&a.bcount[k], s_hist[k]);
 }
 // A shard's draws: all gR global draws are evaluated, a draw's weights block
 // is found from the global block ends, and only draws that land on a local
@@ -430,33 +600,48 @@ __global__ void __launch_bounds__(kDrawThreads) rs_draws_shard_kernel(ResampleAr
 {
     rs_draws_shard_body(a, blockIdx.x * blockDim.x + threadIdx.x);
 }
-__global__ void __launch_bounds__(kDrawThreads) rs_draws_kernel(ResampleArgs a)
+// two draws a thread in large populations: half the flushes of the copy totals
+constexpr int kDrawPer = 2;
+__global__ void __launch_bounds__(kDrawThreads) rs_draws_kernel(ResampleArgs a, int per)
 {
-    rs_draws_body(a, blockIdx.x * blockDim.x + threadIdx.x);
+    rs_draws_body(a, blockIdx.x * blockDim.x * per, per);
 }
 __global__ void __launch_bounds__(kDrawThreads) rs_draws_batched(const ResampleArgs* tab)
 {
     const ResampleArgs& a = tab[blockIdx.y];
     if ((int)(blockIdx.x * blockDim.x) >= a.Rn) return;  // block-uniform: no draw of this instance
-    rs_draws_body(a, blockIdx.x * blockDim.x + threadIdx.x);
+    rs_draws_body(a, blockIdx.x * blockDim.x, 1);
 }
 
 // nearest-integer copy numbers (Sec. II.B, population in expectation):
 // tau_i = target w_i / S, n_i = floor(tau_i) + [u_i < tau_i - floor(tau_i)],
 // u_i from the RESAMPLE stream at counter (i, k, 1)
-__device__ __forceinline__ void rs_nearest_body(const ResampleArgs& a, int i)
+__global__ void __launch_bounds__(256) rs_nearest_kernel(ResampleArgs a)
 {
-    const int R = rs_src(a);
-    if (i >= R) return;
-    const double S = a.cur->S;
-    const u32x4 o = philox((uint32_t)i, (uint32_t)a.k, 1u, a.c3, a.key0, a.key1);
-    const double u = uniform53(o.x, o.y);
-    const double tau = __ddiv_rn(__dmul_rn(a.target, a.w[i]), S);
-    const double fl = floor(tau);
-    a.counts[i] = (int32_t)fl + (u < __dsub_rn(tau, fl) ? 1 : 0);
+    __shared__ int s_n[8];
+    const int R = rs_src(a), i = blockIdx.x * 256 + threadIdx.x;
+    if ((int)blockIdx.x * 256 >= R) return;  // block-uniform
+    int n = 0;
+    if (i < R) {
+        const double S = a.cur->S;
+        const u32x4 o = philox((uint32_t)i, (uint32_t)a.k, 1u, a.c3, a.key0, a.key1);
+        const double u = uniform53(o.x, o.y);
+        const double tau = __ddiv_rn(__dmul_rn(a.target, a.w[i]), S);
+        const double fl = floor(tau);
+        n = (int32_t)fl + (u < __dsub_rn(tau, fl) ? 1 : 0);
+        a.counts[i] = n;
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0) s_n[threadIdx.x >> 5] = n;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        n = __reduce_add_sync(0xffffffffu, threadIdx.x < 8 ? s_n[threadIdx.x] : 0);
+        // 256 replicas lie in one scan block
+        if (threadIdx.x == 0) atomicAdd(&a.bcount[(blockIdx.x * 256) / rs_scan_size(R)], n);
+    }
 }
-__global__ void rs_nearest_kernel(ResampleArgs a) { rs_nearest_body(a, blockIdx.x * blockDim.x + threadIdx.x); }
 
+// ---- copy-number scan and placement of a shard ----
 __device__ __forceinline__ void rs_blocksum_body(const int32_t* counts, int R, int32_t* blocksum, int b)
 {
     __shared__ int ws[32];
@@ -474,17 +659,9 @@ __device__ __forceinline__ void rs_blocksum_body(const int32_t* counts, int R, i
         if (tid == 0) blocksum[b] = v;
     }
 }
-__device__ __forceinline__ void rs_scan_finish(const ResampleArgs& a);
-__global__ void __launch_bounds__(1024) rs_blocksum_kernel(ResampleArgs a)
+__global__ void __launch_bounds__(1024) rs_blocksum_shard_kernel(ResampleArgs a)
 {
-    const int R = rs_src(a);
-    if ((int)blockIdx.x * kScanBlock < R) rs_blocksum_body(a.counts, R, a.blocksum, blockIdx.x);
-    if (a.sync && last_block(a.sync + 1) && threadIdx.x == 0) rs_scan_finish(a);  // block offsets
-}
-__global__ void __launch_bounds__(1024) rs_blocksum_batched(const ResampleArgs* tab)
-{
-    const ResampleArgs& a = tab[blockIdx.y];
-    if ((int)blockIdx.x * kScanBlock < a.R) rs_blocksum_body(a.counts, a.R, a.blocksum, blockIdx.x);
+    rs_blocksum_body(a.counts, a.R, a.blocksum, blockIdx.x);
 }
 
 __device__ __forceinline__ int rs_scan_blocks_body(int32_t* blocksum, int nb)
@@ -497,26 +674,11 @@ __device__ __forceinline__ int rs_scan_blocks_body(int32_t* blocksum, int nb)
     }
     return acc;
 }
-__device__ __forceinline__ void rs_scan_finish(const ResampleArgs& a)
+__global__ void rs_scan_shard_kernel(ResampleArgs a)
 {
-    const int R = rs_src(a);
-    const int nbs = (R + kScanBlock - 1) / kScanBlock;
-    const int total = rs_scan_blocks_body(a.blocksum, nbs);
-    a.blocksum[nbs] = total;  // the copies placed (a shard reads it)
-    if (a.Rdst) {  // the drawn population, copies beyond the capacity dropped
-        const int Rn = min(total, a.cap);
-        *a.Rdst = Rn;
-        *a.Rdst_d = (double)Rn;
-    }
-}
-__global__ void rs_scan_blocks_kernel(ResampleArgs a)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) rs_scan_finish(a);
-}
-__global__ void rs_scan_blocks_batched(const ResampleArgs* tab, int n_inst)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_inst) rs_scan_blocks_body(tab[i].blocksum, (tab[i].R + kScanBlock - 1) / kScanBlock);
+    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    const int nbs = (a.R + kScanBlock - 1) / kScanBlock;
+    a.blocksum[nbs] = rs_scan_blocks_body(a.blocksum, nbs);  // the copies placed
 }
 
 // exclusive scan inside the block + block offset; write parents and families
@@ -571,34 +733,109 @@ __device__ __forceinline__ void rs_fill_body(const ResampleArgs& a, int b)
         }
     }
 }
-__global__ void __launch_bounds__(1024) rs_fill_kernel(ResampleArgs a)
+__global__ void __launch_bounds__(1024) rs_fill_shard_kernel(ResampleArgs a) { rs_fill_body(a, blockIdx.x); }
+
+// Placement: a block takes one scan block of SB replicas.  Its first slot is the
+// sum of the copy totals before it; the inclusive scan of its copy numbers stays
+// in shared memory and every thread takes slots, finding the slot's replica there
+// by bisection, so that a replica with many copies is written by the whole block
+// (one thread per replica took 6.8 ms when one replica filled 10^6 slots).
+// Block 0 also takes the logarithm of S, beside the placement.
+template <int SB>
+__device__ __forceinline__ void rs_place_body(const ResampleArgs& a, int b, int R)
 {
-    if ((int)blockIdx.x * kScanBlock < rs_src(a)) rs_fill_body(a, blockIdx.x);
+    constexpr int PER = SB / 1024;
+    __shared__ int s_cum[SB], s_fam[SB];
+    __shared__ int s_w[32], s_off;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int i0 = b * SB, ns = rs_scan_blocks(R);
+    int c[PER], s = 0, pre = 0, all = 0;
+#pragma unroll
+    for (int t = 0; t < PER; ++t) {
+        const int i = i0 + tid * PER + t;
+        c[t] = i < R ? a.counts[i] : 0;
+        s_fam[tid * PER + t] = i < R ? a.fam_in[i] : 0;
+        s += c[t];
+        c[t] = s;
+    }
+    for (int t = tid; t < ((a.Rdst && b == 0) ? ns : b); t += 1024) {
+        const int v = a.bcount[t];
+        all += v;
+        if (t < b) pre += v;
+    }
+    // inclusive scan of the copy numbers over the block
+    int incl = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    pre = __reduce_add_sync(0xffffffffu, b == 0 ? all : pre);
+    if (lane == 31) s_w[warp] = incl;
+    if (tid == 0) s_off = 0;
+    __syncthreads();
+    if (lane == 0 && pre) atomicAdd(&s_off, pre);
+    int before = lane < warp ? s_w[lane] : 0;
+    before = __reduce_add_sync(0xffffffffu, before);
+#pragma unroll
+    for (int t = 0; t < PER; ++t) {
+        const int i = i0 + tid * PER + t;
+        s_cum[tid * PER + t] = before + incl - s + c[t];
+        if (i < R) a.counts[i] = 0;
+    }
+    __syncthreads();
+    const int total = s_cum[SB - 1], cap = a.Rdst ? a.cap : 0x7fffffff;
+    const int off = b == 0 ? 0 : s_off;
+    if (b == 0 && tid == 0 && a.Rdst) {  // the drawn population, copies beyond the capacity dropped
+        const int Rn = min(s_off, cap);
+        *a.Rdst = Rn;
+        *a.Rdst_d = (double)Rn;
+    }
+    if (b == 0 && tid == 1023) rs_lnq(a);
+    for (int t = tid; t < total && off + t < cap; t += 1024) {
+        int lo = 0, hi = SB - 1;  // the first replica whose inclusive sum exceeds t
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (t < s_cum[mid]) hi = mid; else lo = mid + 1;
+        }
+        a.parent[off + t] = i0 + lo;
+        a.fam_out[off + t] = s_fam[lo];
+    }
 }
-__global__ void __launch_bounds__(1024) rs_fill_batched(const ResampleArgs* tab)
+__device__ __forceinline__ void rs_place_launch(const ResampleArgs& a, int b)
 {
-    const ResampleArgs& a = tab[blockIdx.y];
-    if ((int)blockIdx.x * kScanBlock < a.R) rs_fill_body(a, blockIdx.x);
+    const int R = rs_src(a);
+    if (b >= max(1, rs_scan_blocks(R))) return;  // block-uniform
+    if (rs_scan_size(R) == 1024) rs_place_body<1024>(a, b, R);
+    else rs_place_body<4096>(a, b, R);
 }
+__global__ void __launch_bounds__(1024) rs_place_kernel(ResampleArgs a) { rs_place_launch(a, blockIdx.x); }
+__global__ void __launch_bounds__(1024) rs_place_batched(const ResampleArgs* tab) { rs_place_launch(tab[blockIdx.y], blockIdx.x); }
+
+// blocks that cover the scan blocks of every population up to R: a smaller one
+// (drawn on the device) may have smaller scan blocks
+static int place_grid(int R) { return rs_bcount_size(R); }
 
 cudaError_t launch_resample(const ResampleArgs& a, cudaStream_t st)
 {
-    const int nb = (a.R + kScanBlock - 1) / kScanBlock;
-    // one level per thread, small blocks spread over the SMs (FP64-bound)
-    if (a.wtab) rs_table_kernel<<<(a.wtab_n + 31) / 32, 32, 0, st>>>(a);
-    rs_weights_kernel<<<rs_wblocks(a.R), kWThreads, 0, st>>>(a);
-    if (!a.sync) rs_top_kernel<<<1, kWBlock, 0, st>>>(a);
-    rs_finalize_kernel<<<rs_wblocks(a.R), kWThreads, 0, st>>>(a);
-    if (!a.sync) rs_blockmax_kernel<<<1, kWBlock, 0, st>>>(a);
+    // a.R sizes the grids (the capacity when the population is in device memory)
+    const bool fused = a.R <= kFuseR;
+    if (fused) {
+        rs_weights_fused_kernel<<<rs_wblocks(a.R), kWBlock, 0, st>>>(a);
+    } else {
+        rs_weights_kernel<<<rs_wblocks(a.R), kWThreads, 0, st>>>(a);
+        rs_runs_kernel<<<(rs_wblocks(a.R) + kRunWarps - 1) / kRunWarps, 32 * kRunWarps, 0, st>>>(a);
+    }
     if (a.scheme == 1)
         rs_nearest_kernel<<<(a.R + 255) / 256, 256, 0, st>>>(a);
+    else if (fused)
+        rs_draws_kernel<<<(a.Rn + kDrawSmall - 1) / kDrawSmall, kDrawSmall, 0, st>>>(a, 1);
     else
-        rs_draws_kernel<<<(a.Rn + kDrawThreads - 1) / kDrawThreads, kDrawThreads, 0, st>>>(a);
-    rs_blocksum_kernel<<<nb, 1024, 0, st>>>(a);
-    if (!a.sync) rs_scan_blocks_kernel<<<1, 32, 0, st>>>(a);
-    rs_fill_kernel<<<nb, 1024, 0, st>>>(a);
+        rs_draws_kernel<<<(a.Rn + kDrawPer * kDrawThreads - 1) / (kDrawPer * kDrawThreads), kDrawThreads, 0, st>>>(a, kDrawPer);
+    rs_place_kernel<<<place_grid(a.R), 1024, 0, st>>>(a);
     return cudaGetLastError();
 }
+int resample_launches(const ResampleArgs& a) { return a.R <= kFuseR ? 3 : 4; }
 
 // the phases of a shard's resampling (the host exchanges the block totals,
 // the block maxima and the copy totals between them)
@@ -607,21 +844,20 @@ cudaError_t launch_resample_shard(const ResampleArgs& a, int phase, cudaStream_t
     const int nb = (a.R + kScanBlock - 1) / kScanBlock;
     switch (phase) {
     case 0:  // weights, levels 0 and 1 of the local blocks -> local block totals in upper
-        if (a.wtab) rs_table_kernel<<<(a.wtab_n + 31) / 32, 32, 0, st>>>(a);
-        rs_weights_kernel<<<rs_wblocks(a.R), kWThreads, 0, st>>>(a);
+        rs_weights_shard_kernel<<<rs_wblocks(a.R), kWThreads, 0, st>>>(a);
         break;
     case 1:  // global levels >= 2 (upper holds every shard's block totals), local P, block maxima
         rs_top_kernel<<<1, kWBlock, 0, st>>>(a);
-        rs_finalize_kernel<<<rs_wblocks(a.R), kWThreads, 0, st>>>(a);
+        rs_finalize_shard_kernel<<<rs_wblocks(a.R), kWThreads, 0, st>>>(a);
         break;
     case 2:  // running maximum over every shard's blocks, S, ln Q; draws; copy totals
-        rs_blockmax_kernel<<<1, kWBlock, 0, st>>>(a);
+        rs_blockmax_shard_kernel<<<1, kWBlock, 0, st>>>(a);
         rs_draws_shard_kernel<<<(a.Rn + kDrawThreads - 1) / kDrawThreads, kDrawThreads, 0, st>>>(a);
-        rs_blocksum_kernel<<<nb, 1024, 0, st>>>(a);
-        rs_scan_blocks_kernel<<<1, 32, 0, st>>>(a);
+        rs_blocksum_shard_kernel<<<nb, 1024, 0, st>>>(a);
+        rs_scan_shard_kernel<<<1, 32, 0, st>>>(a);
         break;
     default:  // placement: global parent indices and families of the local copies
-        rs_fill_kernel<<<nb, 1024, 0, st>>>(a);
+        rs_fill_shard_kernel<<<nb, 1024, 0, st>>>(a);
         break;
     }
     return cudaGetLastError();
@@ -629,16 +865,11 @@ cudaError_t launch_resample_shard(const ResampleArgs& a, int phase, cudaStream_t
 
 cudaError_t launch_resample_batched(const ResampleArgs* tab, int n_inst, int maxR, cudaStream_t st)
 {
-    const unsigned nb = (maxR + kScanBlock - 1) / kScanBlock;
     const unsigned ni = (unsigned)n_inst;
     rs_weights_batched<<<dim3(rs_wblocks(maxR), ni), kWThreads, 0, st>>>(tab);
-    rs_top_batched<<<ni, kWBlock, 0, st>>>(tab, n_inst);
-    rs_finalize_batched<<<dim3(rs_wblocks(maxR), ni), kWThreads, 0, st>>>(tab);
-    rs_blockmax_batched<<<ni, kWBlock, 0, st>>>(tab, n_inst);
+    rs_runs_batched<<<dim3((rs_wblocks(maxR) + kRunWarps - 1) / kRunWarps, ni), 32 * kRunWarps, 0, st>>>(tab);
     rs_draws_batched<<<dim3((maxR + kDrawThreads - 1) / kDrawThreads, ni), kDrawThreads, 0, st>>>(tab);
-    rs_blocksum_batched<<<dim3(nb, ni), 1024, 0, st>>>(tab);
-    rs_scan_blocks_batched<<<(ni + 63) / 64, 64, 0, st>>>(tab, n_inst);
-    rs_fill_batched<<<dim3(nb, ni), 1024, 0, st>>>(tab);
+    rs_place_batched<<<dim3(place_grid(maxR), ni), 1024, 0, st>>>(tab);
     return cudaGetLastError();
 }
 
@@ -658,11 +889,16 @@ cudaError_t launch_logc_table(double* t, cudaStream_t st)
 // kObsBlocks blocks each reduce a contiguous slice of the population in a
 // fixed order; one block combines the partials in block order.  The result
 // does not depend on the GPU (the partition depends only on R).
+// The launch is latency: one round of loads, then short chains.  A run of equal
+// family ids ends at the next start, found from the warp's ballot, the other
+// warps' first starts, and only for the last run of a 1024-replica window by a
+// search beyond it (the whole warp, 32 probes a round).
 __device__ __forceinline__ void observe_partial_body(const ObsArgs& a)
 {
     __shared__ long long s_ll[2][32];
     __shared__ double s_d[3][32];
     __shared__ __int128 s_min[32];
+    __shared__ int s_first[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R = a.Rdev ? *a.Rdev : a.R;
     const int nb = obs_blocks(R);
@@ -671,63 +907,85 @@ __device__ __forceinline__ void observe_partial_body(const ObsArgs& a)
     const int j0 = blockIdx.x * per, j1 = min(R, j0 + per);
     long long se = 0, se2 = 0;
     double sed = 0.0, se2d = 0.0, clnc = 0.0;
+    int mn32 = 0x7fffffff;
     __int128 mn = (__int128)(((unsigned __int128)1 << 127) - 1);
-    for (int j = j0 + tid; j < j1; j += 1024) {
-        if (a.kind == 0) {
-            const long long e = a.E32[j];
-            se += e;
-            se2 += e * e;
-            if ((__int128)e < mn) mn = e;
-        } else {
-            const longlong2 v = a.E128[j];
-            const __int128 e = ((__int128)v.y << 64) | (unsigned long long)v.x;
-            const double ed = __dmul_rn(i128_to_double(e), 0x1p-96);
-            sed = __dadd_rn(sed, ed);
-            se2d = __fma_rn(ed, ed, se2d);
-            if (e < mn) mn = e;
+    for (int jb = j0; jb < j1; jb += 1024) {
+        const int j = jb + tid, jend = min(j1, jb + 1024);
+        int f = 0, fprev = 0;
+        if (j < j1) {
+            f = a.family[j];
+            fprev = j > 0 ? a.family[j - 1] : f;
+            if (a.kind == 0) {
+                const int e = a.E32[j];
+                se += e;
+                se2 += (long long)e * e;
+                mn32 = min(mn32, e);
+            } else {
+                const longlong2 v = a.E128[j];
+                const __int128 e = ((__int128)v.y << 64) | (unsigned long long)v.x;
+                const double ed = __dmul_rn(i128_to_double(e), 0x1p-96);
+                sed = __dadd_rn(sed, ed);
+                se2d = __fma_rn(ed, ed, se2d);
+                if (e < mn) mn = e;
+            }
         }
-        const int f = a.family[j];
-        if (j == 0 || a.family[j - 1] != f) {
-            // end of the run of family f (families are sorted): a short
-            // forward look first, bisection for long runs
-            int e = j + 1;
-            while (e < R && e < j + 8 && a.family[e] == f) ++e;
-            if (e < R && a.family[e] == f) {
-                int lo = e + 1, hi = R;  // first index with family > f
+        const bool start = j < j1 && (j == 0 || fprev != f);
+        const unsigned bal = __ballot_sync(0xffffffffu, start);
+        if (lane == 0) s_first[warp] = bal ? jb + warp * 32 + __ffs(bal) - 1 : 0x7fffffff;
+        __syncthreads();
+        if (bal) {  // warp-uniform
+            // first start in a later warp, or beyond the window for the last run
+            int nxt = __reduce_min_sync(0xffffffffu, lane > warp ? s_first[lane] : 0x7fffffff);
+            if (nxt == 0x7fffffff) {
+                const int fl = __shfl_sync(0xffffffffu, f, 31 - __clz(bal));
+                int lo = jend, hi = R;  // the first index in [lo, hi) of another family, else hi
                 while (lo < hi) {
-                    const int mid = lo + ((hi - lo) >> 1);
-                    if (a.family[mid] > f) hi = mid; else lo = mid + 1;
+                    const int step = (hi - lo + 31) / 32, at = lo + lane * step;
+                    const unsigned ne = __ballot_sync(0xffffffffu, at < hi && a.family[at] != fl);
+                    // the end lies after the last equal probe, at or before the first other one
+                    const int k = ne ? __ffs(ne) - 1 : __popc(__ballot_sync(0xffffffffu, at < hi));
+                    const int nlo = k == 0 ? lo : lo + (k - 1) * step + 1;
+                    hi = ne ? lo + k * step : hi;
+                    lo = min(nlo, hi);
                 }
-                e = lo;
+                nxt = lo;
             }
-            // c ln c of the run; a run of one adds exactly 0 (GB300's FP64 log
-            // is costly: short runs read it from the context's table, which
-            // holds the same device log of the same argument)
-            const int cn = e - j;
-            if (cn > 1) {
-                const double c = (double)cn;
-                const double lc = (a.logc && cn < kLogC) ? a.logc[cn] : log(c);
-                clnc = __fma_rn(c, lc, clnc);
+            if (start) {
+                const unsigned later = bal & ~((2u << lane) - 1u);
+                const int e = later ? jb + warp * 32 + __ffs(later) - 1 : nxt;
+                // c ln c of the run; a run of one adds exactly 0 (GB300's FP64 log
+                // is costly: short runs read it from the context's table, which
+                // holds the same device log of the same argument)
+                const int cn = e - j;
+                if (cn > 1) {
+                    const double c = (double)cn;
+                    const double lc = (a.logc && cn < kLogC) ? a.logc[cn] : log(c);
+                    clnc = __fma_rn(c, lc, clnc);
+                }
             }
         }
+        __syncthreads();  // s_first is rewritten by the next window
     }
     // fixed shuffle trees; the FP64 ones only where they can add something
     // (GB300 has little FP64 throughput): +-J energies are integer sums, and a
     // warp without a family start has clnc = 0 in every lane
+    if (a.kind == 0) {
+        mn32 = __reduce_min_sync(0xffffffffu, mn32);
+        mn = mn32;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        se += __shfl_down_sync(0xffffffffu, se, off);
-        se2 += __shfl_down_sync(0xffffffffu, se2, off);
-        const long long lo = __shfl_down_sync(0xffffffffu, (long long)(unsigned long long)mn, off);
-        const long long hi = __shfl_down_sync(0xffffffffu, (long long)(mn >> 64), off);
-        const __int128 o = ((__int128)hi << 64) | (unsigned long long)lo;
-        if (o < mn) mn = o;
-    }
-    if (a.kind != 0) {
+        for (int off = 16; off > 0; off >>= 1) {
+            se += __shfl_down_sync(0xffffffffu, se, off);
+            se2 += __shfl_down_sync(0xffffffffu, se2, off);
+        }
+    } else {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             sed = __dadd_rn(sed, __shfl_down_sync(0xffffffffu, sed, off));
             se2d = __dadd_rn(se2d, __shfl_down_sync(0xffffffffu, se2d, off));
+            const long long lo = __shfl_down_sync(0xffffffffu, (long long)(unsigned long long)mn, off);
+            const long long hi = __shfl_down_sync(0xffffffffu, (long long)(mn >> 64), off);
+            const __int128 o = ((__int128)hi << 64) | (unsigned long long)lo;
+            if (o < mn) mn = o;
         }
     }
     if (__any_sync(0xffffffffu, clnc != 0.0)) {
@@ -740,30 +998,47 @@ __device__ __forceinline__ void observe_partial_body(const ObsArgs& a)
         s_min[warp] = mn;
     }
     __syncthreads();
-    if (tid == 0) {
-        ObsPartial p;
-        p.sumE = 0; p.sumE2 = 0; p.sumEd = 0.0; p.sumE2d = 0.0; p.clnc = 0.0; p.pad = 0.0;
-        __int128 M = s_min[0];
-        for (int w = 0; w < 32; ++w) {
-            p.sumE += s_ll[0][w]; p.sumE2 += s_ll[1][w];
-            p.sumEd = __dadd_rn(p.sumEd, s_d[0][w]); p.sumE2d = __dadd_rn(p.sumE2d, s_d[1][w]);
-            p.clnc = __dadd_rn(p.clnc, s_d[2][w]);
-            if (s_min[w] < M) M = s_min[w];
+    if (warp != 0) return;
+    ObsPartial& p = a.part[blockIdx.x];
+    if (a.kind == 0) {
+        se = s_ll[0][lane]; se2 = s_ll[1][lane];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            se += __shfl_down_sync(0xffffffffu, se, off);
+            se2 += __shfl_down_sync(0xffffffffu, se2, off);
         }
+        const int m = __reduce_min_sync(0xffffffffu, (int)s_min[lane]);
+        if (lane == 0) { p.sumE = se; p.sumE2 = se2; p.min_lo = m; p.min_hi = m < 0 ? -1 : 0; }
+    } else if (lane == 3) {
+        __int128 M = s_min[0];
+        for (int w = 1; w < 32; ++w)
+            if (s_min[w] < M) M = s_min[w];
+        p.sumE = 0; p.sumE2 = 0;
         p.min_lo = (long long)(unsigned long long)M;
         p.min_hi = (long long)(M >> 64);
-        a.part[blockIdx.x] = p;
+    }
+    if (lane < 3) {  // the warps' FP64 sums in warp order, one chain per lane (+0 first: no change)
+        double acc = 0.0;
+        if (lane == 2 || a.kind != 0)
+            for (int w = 0; w < 32; ++w) acc = __dadd_rn(acc, s_d[lane][w]);
+        if (lane == 0) p.sumEd = acc;
+        else if (lane == 1) p.sumE2d = acc;
+        else p.clnc = acc;
     }
 }
 __device__ __forceinline__ void observe_final_body(const ObsArgs& a);
 __global__ void __launch_bounds__(1024) observe_partial_kernel(ObsArgs a)
 {
     observe_partial_body(a);
-    if (a.sync && last_block(a.sync) && threadIdx.x < 32) observe_final_body(a);  // combine in a fixed order
+    const int nb = obs_blocks(a.Rdev ? *a.Rdev : a.R);
+    if ((int)blockIdx.x < nb && last_block(a.sync, nb) && threadIdx.x < 32) observe_final_body(a);  // combine in a fixed order
 }
 __global__ void __launch_bounds__(1024) observe_partial_batched(const ObsArgs* tab)
 {
-    observe_partial_body(tab[blockIdx.y]);
+    const ObsArgs& a = tab[blockIdx.y];
+    observe_partial_body(a);
+    const int nb = obs_blocks(a.R);
+    if ((int)blockIdx.x < nb && last_block(a.sync, nb) && threadIdx.x < 32) observe_final_body(a);
 }
 
 // partials combined by one warp: lane l adds blocks l, l + 32, ... in order,
@@ -802,28 +1077,15 @@ __device__ __forceinline__ void observe_final_body(const ObsArgs& a)
     a.cur->emin_lo = (long long)(unsigned long long)M;
     a.cur->emin_hi = (long long)(M >> 64);
 }
-__global__ void observe_final_kernel(ObsArgs a)
-{
-    if (threadIdx.x < 32) observe_final_body(a);
-}
-// one warp per instance
-__global__ void observe_final_batched(const ObsArgs* tab, int n_inst)
-{
-    const int i = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    if (i < n_inst) observe_final_body(tab[i]);
-}
-
 cudaError_t launch_observe(const ObsArgs& a, cudaStream_t st)
 {
     observe_partial_kernel<<<obs_blocks(a.R), 1024, 0, st>>>(a);
-    if (!a.sync) observe_final_kernel<<<1, 32, 0, st>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_observe_batched(const ObsArgs* tab, int n_inst, int maxR, cudaStream_t st)
 {
     observe_partial_batched<<<dim3(obs_blocks(maxR), (unsigned)n_inst), 1024, 0, st>>>(tab);
-    observe_final_batched<<<(n_inst + 7) / 8, 256, 0, st>>>(tab, n_inst);
     return cudaGetLastError();
 }
 
