@@ -7,17 +7,25 @@
 
 namespace pa {
 
+// Block b takes GPB groups; with `spread` the groups are spread evenly over the
+// grid instead (at most GPB a block).
 template <int D, int L, int GPB, int THREADS, bool I8, bool SHARD = false>
-__global__ void __launch_bounds__(THREADS, 4) sweep_packed_kernel(PackedSweepArgs a)
+__global__ void __launch_bounds__(THREADS, 4) sweep_packed_kernel(PackedSweepArgs a, int spread)
 {
     extern __shared__ __align__(16) unsigned char smem_packed[];
-    sweep_packed_tile<D, L, GPB, THREADS, I8, true, SHARD>(a.s, a.i, blockIdx.x * GPB, smem_packed);
+    const int G = packed_groups(a.i);
+    int g0 = blockIdx.x * GPB, gend = min(g0 + GPB, G);
+    if (GPB > 1 && spread) {
+        g0 = (int)((long long)G * blockIdx.x / gridDim.x);
+        gend = (int)((long long)G * (blockIdx.x + 1) / gridDim.x);
+    }
+    sweep_packed_tile<D, L, GPB, THREADS, I8, true, SHARD>(a.s, a.i, g0, gend, smem_packed);
 }
 
 // ---------------- shapes and dispatch ----------------
 
 template <int D, int L, int GPB, int THREADS, bool I8, bool SHARD = false>
-static cudaError_t launch_one(const PackedSweepArgs& a, cudaStream_t st)
+static cudaError_t launch_one(const PackedSweepArgs& a, int grid, int spread, cudaStream_t st)
 {
     const size_t smem = PackedShape<D, L, GPB, THREADS>::SMEM;
     auto kern = sweep_packed_kernel<D, L, GPB, THREADS, I8, SHARD>;
@@ -27,8 +35,7 @@ static cudaError_t launch_one(const PackedSweepArgs& a, cudaStream_t st)
         if (e != cudaSuccess) return e;
         attr_done = true;
     }
-    int grid = (a.i.G + GPB - 1) / GPB;
-    kern<<<grid, THREADS, smem, st>>>(a);
+    kern<<<grid, THREADS, smem, st>>>(a, spread);
     return cudaGetLastError();
 }
 
@@ -37,17 +44,32 @@ static cudaError_t launch_dl(const PackedSweepArgs& a, int gpb, int threads, cud
 {
     constexpr Shape s = default_shape<D, L>();
     const bool i8 = a.i.S8_out != nullptr;
+    int grid = (a.i.G + gpb - 1) / gpb;
     if (a.i.goff != 0) {  // a shard (packed words, default shape)
         if (i8 || gpb != s.gpb || threads != s.threads) return cudaErrorInvalidConfiguration;
-        return launch_one<D, L, s.gpb, s.threads, false, true>(a, st);
+        return launch_one<D, L, s.gpb, s.threads, false, true>(a, grid, 0, st);
     }
     // the one tuned alternative: twice the groups per block, same thread count
     if (gpb == 2 * s.gpb && threads == s.threads)
-        return i8 ? launch_one<D, L, 2 * s.gpb, s.threads, true>(a, st)
-                  : launch_one<D, L, 2 * s.gpb, s.threads, false>(a, st);
+        return i8 ? launch_one<D, L, 2 * s.gpb, s.threads, true>(a, grid, 0, st)
+                  : launch_one<D, L, 2 * s.gpb, s.threads, false>(a, grid, 0, st);
     if (gpb != s.gpb || threads != s.threads) return cudaErrorInvalidConfiguration;
-    return i8 ? launch_one<D, L, s.gpb, s.threads, true>(a, st)
-              : launch_one<D, L, s.gpb, s.threads, false>(a, st);
+    // fewer than two full blocks to an SM: spread the groups over up to four
+    // blocks to an SM (L=6, R=40001: 119 -> 81 us; L=6, R=5000: 116 -> 41 us;
+    // 2D L=16, R=30000: 125 -> 68 us); with more full blocks than that spreading
+    // measured 2 to 5 % slower (L=8, R=10^5: 213 -> 218 us)
+    int spread = 0;
+    if constexpr (s.gpb > 1) {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (grid < 2 * sms) {
+            spread = 1;
+            grid = a.i.G < 4 * sms ? a.i.G : 4 * sms;
+        }
+    }
+    return i8 ? launch_one<D, L, s.gpb, s.threads, true>(a, grid, spread, st)
+              : launch_one<D, L, s.gpb, s.threads, false>(a, grid, spread, st);
 }
 
 // launch for the lattice sizes of one part: *handled is false when (D, L)

@@ -47,6 +47,18 @@ __device__ __forceinline__ int site_parity(int i)
     return (x + y + z) & 1;
 }
 
+// 32x32 bit matrix transpose across a warp: lane l's bit k becomes lane k's bit l
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane)
+{
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const uint32_t m = s == 16 ? 0x0000FFFFu : s == 8 ? 0x00FF00FFu : s == 4 ? 0x0F0F0F0Fu : s == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
+        x = (lane & s) ? ((y >> s) & m) | (x & ~m) : (x & m) | ((y << s) & ~m);
+    }
+    return x;
+}
+
 // a 0 / ~0 32-bit mask widened to 64 bits (both halves the same register)
 __device__ __forceinline__ uint64_t rep32(uint32_t v) { return ((uint64_t)v << 32) | v; }
 
@@ -115,6 +127,12 @@ struct Shape {
     int gpb, threads;
 };
 
+// the population's groups (in device memory for the nearest-integer scheme)
+__device__ __forceinline__ int packed_groups(const PackedInst& in)
+{
+    return in.Rdev ? (__ldg(in.Rdev) + 63) >> 6 : in.G;
+}
+
 // default groups per block and threads of the packed sweep for a lattice
 template <int D, int L> __host__ __device__ constexpr Shape default_shape()
 {
@@ -127,14 +145,14 @@ template <int D, int L> __host__ __device__ constexpr Shape default_shape()
          : Shape{1, 256};
 }
 
-// groups [g0, g0 + GPB) of one instance; smem holds PackedShape::SMEM bytes
+// groups [g0, gend) of one instance, at most GPB; smem holds PackedShape::SMEM bytes
 // LATE: allow the late compaction of modes 0 and 2 (the single-instance
 // kernels; the disorder batch measured slower with it)
 // SHARD: the instance is a shard of a larger population; its PLANE counters
 // carry the global group index g0 + in.goff (a separate instantiation, so
 // that the counters of every other launch cost nothing extra)
 template <int D, int L, int GPB, int THREADS, bool I8, bool LATE = true, bool SHARD = false>
-__device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const PackedInst& in, int g0,
+__device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const PackedInst& in, int g0, int gend,
                                                   unsigned char* smem)
 {
     using LT = Lat<D, L>;
@@ -147,8 +165,7 @@ __device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const Pac
     unsigned char* qbuf = smem + SH::TILE + SH::SJ + SH::CNT;
 
     const int R = in.Rdev ? __ldg(in.Rdev) : in.R;
-    const int G = in.Rdev ? (R + 63) >> 6 : in.G;
-    if (g0 >= G) return;  // block-uniform: past the population held in device memory
+    if (g0 >= gend) return;  // block-uniform: past the population held in device memory
     const uint32_t c3 = in.c3;
     // a shard's groups carry their global index in the PLANE counters:
     // 16 goff added to counter word 2 through its first-round product
@@ -162,11 +179,12 @@ __device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const Pac
     // first-round products that depend on it alone off the vector pipes:
     // L=16, k=5..24: 2837 -> 2875 attempts/ns)
     const int32_t* __restrict__ parent = in.parent;
-    const int ng = GPB == 1 ? 1 : min(GPB, G - g0);  // g0 < G: one group is always full
+    const int ng = GPB == 1 ? 1 : min(GPB, gend - g0);
     const int tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
 
-    for (int t = tid; t < N; t += THREADS) sj[t] = in.jneg[t];
+    // coupling signs in sublattice order
+    for (int t = tid; t < N; t += THREADS) sj[site_parity<D, L>(t) * NH + (t >> 1)] = in.jneg[t];
 
     if (!I8 && !parent) {
         for (int t = tid; t < ng * N; t += THREADS) {
@@ -177,27 +195,37 @@ __device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const Pac
     } else if (!I8) {
         // fused resampling gather: lane j of group g takes the bit of replica
         // parent[64g+j]; parents are non-decreasing, so the 64 sources of a word
-        // sit in one to a few neighbouring groups.  Each thread owns destination
-        // lanes `lane` and `lane+32`; two ballots assemble a word; the word of
-        // site base+t is kept by lane t and stored once per 32 sites.
+        // sit in one to a few neighbouring groups.  A lane collects the bits of
+        // its two destination replicas (lane, lane + 32) over 32 sites, two
+        // shifts a site from the 32-bit half of the source word that holds them;
+        // two transposes across the warp then give lane t the word of site
+        // base + t.  Two ballots a site and a select took twice the instructions
+        // (L=16, R=10^5, a launch without sweeps: 178 -> 143 us, with ten
+        // 1294 -> 1258 us).
         constexpr int NCH = (N + 31) / 32;
         for (int tup = warp; tup < ng * NCH; tup += NWARP) {
             const int gl = tup / NCH, base = (tup - gl * NCH) * 32;
             const int r0 = 64 * (g0 + gl) + lane, r1 = r0 + 32;
             const int s0 = r0 < R ? parent[r0] : r0;
             const int s1 = r1 < R ? parent[r1] : r1;
-            const uint64_t* p0 = in.Sin + (size_t)(s0 >> 6) * N + base;
-            const uint64_t* p1 = in.Sin + (size_t)(s1 >> 6) * N + base;
-            const int sb0 = s0 & 63, sb1 = s1 & 63;
+            const uint32_t* p0 = reinterpret_cast<const uint32_t*>(in.Sin + (size_t)(s0 >> 6) * N + base) + ((s0 >> 5) & 1);
+            const uint32_t* p1 = reinterpret_cast<const uint32_t*>(in.Sin + (size_t)(s1 >> 6) * N + base) + ((s1 >> 5) & 1);
+            const int sb0 = s0 & 31, sb1 = s1 & 31;
             const int cnt32 = min(32, N - base);
-            uint64_t mine = 0;
-#pragma unroll 4
-            for (int t = 0; t < cnt32; ++t) {
-                const uint64_t w0 = __ldg(p0 + t), w1 = __ldg(p1 + t);
-                const uint32_t lo = __ballot_sync(0xffffffffu, (uint32_t)(w0 >> sb0) & 1u);
-                const uint32_t hi = __ballot_sync(0xffffffffu, (uint32_t)(w1 >> sb1) & 1u);
-                if (lane == t) mine = (uint64_t)lo | ((uint64_t)hi << 32);
+            uint32_t a0 = 0, a1 = 0;
+            if (cnt32 == 32) {
+#pragma unroll 8
+                for (int t = 0; t < 32; ++t) {
+                    a0 = __funnelshift_r(a0, __ldg(p0 + 2 * t) >> sb0, 1);
+                    a1 = __funnelshift_r(a1, __ldg(p1 + 2 * t) >> sb1, 1);
+                }
+            } else {
+                for (int t = 0; t < cnt32; ++t) {
+                    a0 |= ((__ldg(p0 + 2 * t) >> sb0) & 1u) << t;
+                    a1 |= ((__ldg(p1 + 2 * t) >> sb1) & 1u) << t;
+                }
             }
+            const uint64_t mine = (uint64_t)transpose32(a0, lane) | ((uint64_t)transpose32(a1, lane) << 32);
             const int i = base + lane;
             if (lane < cnt32) sm[(gl * 2 + site_parity<D, L>(i)) * NH + (i >> 1)] = mine;
         }
@@ -233,27 +261,10 @@ __device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const Pac
 
     // this thread's x-y column (used when every item of the thread shares it)
     const int xh_c = (tid % NH) % LT::LH, y_c = ((tid % NH) / LT::LH) % L;
-    // item t = (group gl, sublattice index q) of parity p: neighbour decoding,
-    // unsatisfied-bond counts n = b0 + 2 b1 + 4 b2 per lane, lanes with dE <= 0
-    auto classify = [&](int t, int p, const typename LT::Nb& nb_fixed, uint64_t*& cur, int& q,
-                        uint64_t& sw0, uint64_t& b0, uint64_t& b1, uint64_t& b2, uint64_t& down) {
-        const int gl = t / NH;
-        q = t - gl * NH;
-        cur = sm + (gl * 2 + p) * NH;
-        const uint64_t* oth = sm + (gl * 2 + (p ^ 1)) * NH;
-        typename LT::Nb nb;
-        // when every item of this thread sits on the same sublattice site
-        // (THREADS a multiple of N/2) decode once; when it sits on the same x-y
-        // column (3D, THREADS a multiple of L^2/2) only z moves
-        if constexpr (THREADS % NH == 0) {
-            nb = nb_fixed;
-        } else if constexpr (D == 3 && THREADS % (LT::LH * L) == 0) {
-            nb = LT::neighbours_column(p, q, xh_c, y_c);
-        } else {
-            nb = LT::neighbours(p, q);
-        }
-        sw0 = cur[q];
-        const uint32_t jm = sj[nb.site];
+    // unsatisfied-bond counts n = b0 + 2 b1 + 4 b2 per lane of site (p, q), and
+    // lanes with dE <= 0, from the six (four) neighbour words
+    auto count_bonds = [&](uint64_t sw0, const uint64_t* oth, const int* nq, uint32_t jm, uint64_t& b0,
+                           uint64_t& b1, uint64_t& b2, uint64_t& down) {
         uint64_t u[2 * D];
         // bond signs moved to bit 7 of bytes 0..5 of (ja, jb) by two multiplies
         // (the shifted copies do not overlap), then replicated over a word by
@@ -263,7 +274,7 @@ __device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const Pac
         for (int kk = 0; kk < 2 * D; ++kk) {
             uint32_t m32;
             asm("prmt.b32 %0, %1, %2, %3;" : "=r"(m32) : "r"(ja), "r"(jb), "r"((uint32_t)(8 | kk) * 0x1111u));
-            u[kk] = sw0 ^ oth[nb.q[kk]] ^ (((uint64_t)m32 << 32) | m32);
+            u[kk] = sw0 ^ oth[nq[kk]] ^ (((uint64_t)m32 << 32) | m32);
         }
         if (D == 3) {
             uint64_t s1 = u[0] ^ u[1] ^ u[2], c1 = maj3(u[0], u[1], u[2]);
@@ -281,6 +292,28 @@ __device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const Pac
             b2 = c1 & k0;
             down = b1 | b2;         // n >= 2: dE <= 0
         }
+    };
+    // item t = (group gl, sublattice index q) of parity p
+    auto classify = [&](int t, int p, const typename LT::Nb& nb_fixed, uint64_t*& cur, int& q,
+                        uint64_t& sw0, uint64_t& b0, uint64_t& b1, uint64_t& b2, uint64_t& down) {
+        const int gl = t / NH;
+        q = t - gl * NH;
+        cur = sm + (gl * 2 + p) * NH;
+        const uint64_t* oth = sm + (gl * 2 + (p ^ 1)) * NH;
+        sw0 = cur[q];
+        const uint32_t jm = sj[p * NH + q];
+        typename LT::Nb nb;
+        // when every item of this thread sits on the same sublattice site
+        // (THREADS a multiple of N/2) decode once; when it sits on the same x-y
+        // column (3D, THREADS a multiple of L^2/2) only z moves
+        if constexpr (THREADS % NH == 0) {
+            nb = nb_fixed;
+        } else if constexpr (D == 3 && THREADS % (LT::LH * L) == 0) {
+            nb = LT::neighbours_column(p, q, xh_c, y_c);
+        } else {
+            nb = LT::neighbours(p, q);
+        }
+        count_bonds(sw0, oth, nb.q, jm, b0, b1, b2, down);
     };
     // MSB-first comparison r < thr over the planes still needed, per mode
     // (s.mode is uniform over the launch; mode 1 runs on the compacted queue):
@@ -563,40 +596,30 @@ __device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const Pac
     // ---- energies: vertical counters of unsatisfied bonds ----
     {
         const int gl = tid / TPG, lt = tid - gl * TPG;
-        // a thread counts at most ceil(N / TPG) sites of D bonds each
-        constexpr int W = bits_for(((N + TPG - 1) / TPG) * D) > 2 ? bits_for(((N + TPG - 1) / TPG) * D) : 2;
-        static_assert(W <= B, "per-thread counter fits the block counter");
+        // every bond has one site of parity 0: a thread counts the 2D bonds of at
+        // most ceil(NH / TPG) of them (half the words of counting every site's
+        // +e_d bonds; without sweeps 143 -> 137 us)
+        constexpr int W = bits_for(((NH + TPG - 1) / TPG) * 2 * D) > 3 ? bits_for(((NH + TPG - 1) / TPG) * 2 * D) : 3;
+        constexpr int WB = W < B ? W : B;
         uint64_t C[B];
 #pragma unroll
         for (int b = 0; b < B; ++b) C[b] = 0;
         if (gl < ng) {
             const uint64_t* base = sm + gl * 2 * NH;
-            for (int i = lt; i < N; i += TPG) {
-                const int x = i % L, y = (i / L) % L, z = (D == 3) ? i / (L * L) : 0;
-                const int p = (x + y + z) & 1;
-                const uint64_t si = base[p * NH + (i >> 1)];
-                const uint32_t jm = sj[i];
-                int nbs[3];
-                nbs[0] = i - x + (x == L - 1 ? 0 : x + 1);
-                nbs[1] = i + ((y == L - 1) ? -(L - 1) * L : L);
-                if (D == 3) nbs[2] = i + ((z == L - 1) ? -(L - 1) * L * L : L * L);
-                uint64_t ub[3] = {0, 0, 0};  // unsatisfied +e_d bonds of site i
+            for (int q = lt; q < NH; q += TPG) {
+                const auto nb = LT::neighbours(0, q);
+                uint64_t b0, b1, b2, down;
+                count_bonds(base[q], base + NH, nb.q, sj[q], b0, b1, b2, down);
+                // the count (0..2D) added into the thread's counter, whose width
+                // covers this thread's sites only
+                uint64_t carry = C[0] & b0;
+                C[0] ^= b0;
+                uint64_t c2 = maj3(C[1], b1, carry);
+                C[1] ^= b1 ^ carry;
+                carry = maj3(C[2], b2, c2);
+                C[2] ^= b2 ^ c2;
 #pragma unroll
-                for (int d = 0; d < D; ++d) {
-                    const int j = nbs[d];
-                    const uint64_t sjw = base[(p ^ 1) * NH + (j >> 1)];
-                    ub[d] = si ^ sjw ^ (((jm >> (2 * d + 1)) & 1u) ? ~0ull : 0ull);
-                }
-                // the site's count (0..D) as two bit-sliced bits, added into the
-                // thread's counter, whose width W covers this thread's sites only
-                const uint64_t lo = ub[0] ^ ub[1] ^ ub[2], hi = maj3(ub[0], ub[1], ub[2]);
-                uint64_t carry = C[0] & lo;
-                C[0] ^= lo;
-                uint64_t c2 = maj3(C[1], hi, carry);
-                C[1] ^= hi ^ carry;
-                carry = c2;
-#pragma unroll
-                for (int b = 2; b < W; ++b) {
+                for (int b = 3; b < WB; ++b) {
                     const uint64_t tt = C[b] & carry;
                     C[b] ^= carry;
                     carry = tt;
