@@ -751,6 +751,10 @@ static void plan_step(pa_ctx* c, StepPlan* pl)
         ic.k = k; ic.t = 0;
         ic.key0 = k0; ic.key1 = k1; ic.c3 = pa::counter3(pa::STREAM_ICM, c->tag, c->inst);
         ic.err = c->icm_err;
+        // scratch that nothing else uses between the two sweep launches: the
+        // weights (two ints per replica) and the getters' byte buffer (N bytes
+        // per replica, a bit row takes at most that)
+        ic.perm = (int*)c->w; ic.rows = (uint32_t*)c->tmp8;
         if (c->layout != PA_LAYOUT_PACKED || c->kind == PA_REAL) c->cur ^= 1;  // the second sweep launch ping-pongs
     }
     if (c->sep_gather && k > 0) {
@@ -841,16 +845,13 @@ static int enqueue_step(pa_ctx* c)
         PA_CK(c, pa::launch_sweep_real(c->D, c->L, pl.re, c->real_warps, 0, c->st));
     c->launches += 1;
     if (pl.icm) {
-        for (int t = 0; t < 2; ++t) {
-            pa::IcmArgs ic = pl.ic;
-            ic.t = t;
-            PA_CK(c, pa::launch_icm(ic, c->st));
-        }
+        int n_icm = 0;
+        PA_CK(c, pa::launch_icm(pl.ic, &n_icm, c->st));
         if (c->kind == PA_PM1)
             PA_CK(c, pa::launch_sweep_packed(c->D, c->L, pl.pk2, c->gpb, c->threads, c->st));
         else
             PA_CK(c, pa::launch_sweep_real(c->D, c->L, pl.re2, c->real_warps, 0, c->st));
-        c->launches += 3;
+        c->launches += n_icm + 1;
     }
     if (pl.grad_pm) {
         const bool dyn = c->scheme == PA_RESAMPLE_NEAREST;

@@ -148,11 +148,13 @@ struct IcmArgs {
     int8_t* S8;              // int8 rows [R][NP] (or null)
     const int* Rdev;         // population in device memory (or null: R)
     int R;                   // population, or the capacity with Rdev
-    int k, t;                // step, round (0 or 1)
+    int k, t;                // step, round (0 or 1; set per launch)
+    int* perm;               // [2][R] scratch: both rounds' pairings
+    uint32_t* rows;          // packed words: [R][(N + 31) / 32] scratch, a bit row per replica
     uint32_t key0, key1, c3; // Philox key, counter word 3 of the ICM stream
     int* err;                // set if a bounded union-find loop gave up
 };
-cudaError_t launch_icm(const IcmArgs& a, cudaStream_t st);
+cudaError_t launch_icm(const IcmArgs& a, int* launches, cudaStream_t st);
 
 // ---------------- resampling and observables ----------------
 struct ResampleArgs {
