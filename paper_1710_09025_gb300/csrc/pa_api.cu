@@ -34,6 +34,7 @@ struct pa_ctx {
     int gpb, threads, real_warps;
     int band;                   // real couplings: acceptance guard band verified on this device
     int field;                  // some h is not zero (after the flush)
+    int eshift;                 // real couplings: energies fit 64 bits in units of 2^(eshift - 96), or -1
     double betaF0, log_R;
     std::vector<double> betas;
     std::vector<int> Rk;        // population (target) at each temperature; R = capacity
@@ -424,7 +425,7 @@ static int create_impl(pa_ctx** out, int D, int L, int kind, const float* J, con
             c->hh[i] = flush73(h[i]);
             nflush += (c->hh[i] != h[i]);
         }
-    c->field = 0;
+    c->field = 0; c->eshift = -1;
     for (int i = 0; i < N; ++i) c->field |= c->hh[i] != 0.0f;
     if (nflush) c->err = "warning: " + std::to_string(nflush) + " coupling/field magnitudes below 2^-73 flushed to 0";
 
@@ -502,6 +503,19 @@ static int create_impl(pa_ctx** out, int D, int L, int kind, const float* J, con
         hf.resize(N);
         for (int b = 0; b < D * N; ++b) jf[b] = fix96(c->Jh[b]);
         for (int i = 0; i < N; ++i) hf[i] = fix96(c->hh[i]);
+        // the largest energy, sum |J| + sum |h|, and the bit all values share
+        unsigned __int128 sum = 0, any = 0;
+        auto take = [&](const longlong2& v) {
+            const __int128 x = ((__int128)v.y << 64) | (unsigned long long)v.x;
+            const unsigned __int128 m = x < 0 ? (unsigned __int128)(-x) : (unsigned __int128)x;
+            sum += m;
+            any |= m;
+        };
+        for (const auto& v : jf) take(v);
+        for (const auto& v : hf) take(v);
+        int tz = 0;
+        while (tz < 127 && any != 0 && !((any >> tz) & 1)) ++tz;
+        c->eshift = any == 0 ? 0 : (sum >> tz) < ((unsigned __int128)1 << 62) ? tz : -1;
     }
     int rc2 = PA_OK;
     auto up = [&](void* dst, const void* src, size_t n) {
@@ -724,7 +738,7 @@ static void plan_step(pa_ctx* c, StepPlan* pl)
         pa::RealInst& in = pl->re.i;
         in.Sin = c->S8[c->cur]; in.Sout = c->S8[c->cur ^ 1];
         in.parent = k > 0 ? c->parent : nullptr;
-        in.field = c->field;
+        in.field = c->field; in.eshift = c->eshift;
         in.J = c->J; in.h = c->h; in.Jfix = c->Jfix; in.hfix = c->hfix; in.E = c->E128;
         in.cJ = c->acc_grad ? c->cJ + (size_t)k * c->D * c->N : nullptr;
         in.ch = c->acc_grad ? c->ch + (size_t)k * c->N : nullptr;

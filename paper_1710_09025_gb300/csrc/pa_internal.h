@@ -98,6 +98,8 @@ struct RealInst {
     int R, NP;
     uint32_t c3;             // Philox counter word 3 of the WORD stream
     int field;               // some h is not zero
+    int eshift;              // >= 0: every Jfix and hfix is a multiple of 2^eshift and the sum of
+                             // their magnitudes is below 2^(62 + eshift); -1: not so
 };
 struct RealSweepArgs {
     RealStep s;
@@ -197,12 +199,6 @@ struct ResampleArgs {
     int32_t* bcount;             // [rs_scan_blocks] copies per scan block
     int32_t* blocksum;           // a shard: scratch for the count scan
     double* lnQ_out;             // ln Q once more (or null)
-    int32_t* parent;             // [R] out
-    const int32_t* fam_in;       // [R]
-    int32_t* fam_out;            // [R]
-    double dbeta, log_R, betaF0;
-    int k;
-    uint32_t key0, key1, c3;
 };
 // Weight prefix in a fixed order of fan-out kFan: runs of kFan weights summed
 // left to right, the run totals likewise, recursively; each weights block

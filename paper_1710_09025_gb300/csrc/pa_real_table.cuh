@@ -22,9 +22,9 @@
 // stream: the four sites of a quad, one replica) with 34 of them; four replicas
 // of a quad take about 285, 18 per attempt.  Field, exponential and guard band
 // per attempt took 86.  Gaussian couplings, N_S = 10, sweep time per
-// temperature before -> now: 3D L = 10, R = 20000 760 -> 247 us; 3D L = 6,
-// R = 50000 with gradient counts 388 -> 156 us; 2D L = 4 with a field,
-// R = 50000 43 -> 27 us.
+// temperature before -> now: 3D L = 10, R = 20000 760 -> 231 us; 3D L = 6,
+// R = 50000 with gradient counts 388 -> 148 us; 2D L = 4 with a field,
+// R = 50000 43 -> 25 us.
 //
 // Spins are bits: plane w holds 32 replicas in one word per site; replica
 // 4 j + b of the plane is bit 8 b + j, so that four replicas of one group j sit
@@ -148,27 +148,32 @@ __device__ __forceinline__ void tab_couplings(const RealInst& in, int p, int q, 
     for (int k = 0; k < 2 * D; ++k) J[k] = __ldg(in.J + (k >> 1) * LT::N + ((k & 1) ? nb.site : nb.site_m[k >> 1]));
     h = FIELD ? __ldg(in.h + nb.site) : 0.0f;
 }
-// x = f32(beta) dE of the pattern m (bit k: neighbour k is -1) for the own spin +1
-template <int D>
-__device__ __forceinline__ float tab_rule(const float (&J)[2 * D], float h, float beta, uint32_t m)
+// J with the sign of pattern bit k
+__device__ __forceinline__ float tab_term(float J, uint32_t m, int k)
 {
-    float f = 0.0f;
+    return __uint_as_float(__float_as_uint(J) ^ (((m >> k) & 1u) << 31));
+}
+// f summed over the first K neighbours of pattern m (bit k: neighbour k is -1)
+template <int K, int NB>
+__device__ __forceinline__ float tab_sum(const float (&J)[NB], uint32_t m)
+{
+    float f = tab_term(J[0], m, 0);
 #pragma unroll
-    for (int k = 0; k < 2 * D; ++k) {
-        const float tk = __uint_as_float(__float_as_uint(J[k]) ^ (((m >> k) & 1u) << 31));
-        f = k == 0 ? tk : add32(f, tk);
-    }
-    return mul32(beta, mul32(add32(f, h), 2.0f));
+    for (int k = 1; k < K; ++k) f = add32(f, tab_term(J[k], m, k));
+    return f;
 }
 
-// thresholds of every site and pattern at this temperature
+// thresholds of every site and pattern at this temperature.  The sums over the
+// first three neighbours are kept for the patterns that share them.
 template <int D, int L, bool FIELD>
 __device__ __forceinline__ void tab_stage_thresholds(const RealInst& in, float beta, unsigned char* smem)
 {
     using SH = TabShape<D, L, FIELD>;
     constexpr int NPAT = 1 << SH::KI;                    // neighbour patterns
     constexpr int NCOL = 2 * 4 * SH::NBLK * 32;          // table columns (sites)
-    constexpr int SPLIT = NCOL >= kTabThreads ? 1 : 8;   // threads per column
+    // threads per column: with eight, each takes one pattern of the first three neighbours
+    constexpr int SPLIT = NCOL >= kTabThreads ? 1 : 8;
+    constexpr int LOW = 8 / SPLIT;
     for (int it = threadIdx.x; it < NCOL * SPLIT; it += kTabThreads) {
         const int lane = it & 31, c = (it >> 5) % (NCOL / 32), part = it / NCOL;
         const int blk = c % SH::NBLK, t = (c / SH::NBLK) & 3, p = c / (4 * SH::NBLK);
@@ -176,25 +181,37 @@ __device__ __forceinline__ void tab_stage_thresholds(const RealInst& in, float b
         unsigned char* col = smem + (size_t)(p * SH::NBLK + blk) * SH::BLOCK + SH::tpart(t) + lane * 4;
         const bool valid = q < SH::NH;
         float J[2 * D], h = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 2 * D; ++k) J[k] = 0.0f;
         if (valid) tab_couplings<D, L, FIELD>(in, p, q, J, h);
-        for (uint32_t m = part * (NPAT / SPLIT); m < (part + 1) * (NPAT / SPLIT); ++m) {
+        float s3[LOW];
+#pragma unroll
+        for (int i = 0; i < LOW; ++i) s3[i] = tab_sum<3>(J, (uint32_t)(SPLIT == 1 ? i : part));
+#pragma unroll 1
+        for (uint32_t hi = 0; hi < NPAT / 8; ++hi) {
             // without a field bit 2D - 1 of m is 0: the last neighbour is +1
-            uint32_t up = 0u, down = 0u;  // the padding's spins never flip
-            bool pos = false;
-            if (valid) {
+            float t3[2 * D];
+#pragma unroll
+            for (int k = 3; k < 2 * D; ++k) t3[k] = tab_term(J[k], hi << 3, k);
+#pragma unroll
+            for (int i = 0; i < LOW; ++i) {
+                const uint32_t m = (hi << 3) | (uint32_t)(SPLIT == 1 ? i : part);
+                float f = s3[i];
+#pragma unroll
+                for (int k = 3; k < 2 * D; ++k) f = add32(f, t3[k]);
                 // uphill for the spin +1 if x > 0, else for the spin -1 (or free)
-                const float x = tab_rule<D>(J, h, beta, m);
-                pos = x > 0.0f;
+                const float x = mul32(beta, mul32(add32(f, h), 2.0f));
+                const bool pos = x > 0.0f;
                 const float e = spec_expf(fminf(-fabsf(x), 0.0f));
-                up = e == 1.0f ? 0xFFFFFFFFu : __float2uint_rz(mul32(e, 4294967296.0f));
-                down = 0xFFFFFFFFu;
-            }
-            if constexpr (SH::WIDE) {
-                *reinterpret_cast<uint32_t*>(col + m * 256) = pos ? up : down;
-                *reinterpret_cast<uint32_t*>(col + (m + NPAT) * 256) = pos ? down : up;
-            } else {
-                *reinterpret_cast<uint16_t*>(col + m * 256) = (uint16_t)((pos ? up : down) >> 16);
-                *reinterpret_cast<uint16_t*>(col + (m + NPAT) * 256) = (uint16_t)((pos ? down : up) >> 16);
+                uint32_t up = e == 1.0f ? 0xFFFFFFFFu : __float2uint_rz(mul32(e, 4294967296.0f)), down = 0xFFFFFFFFu;
+                if (!valid) up = down = 0u;  // the padding's spins never flip
+                if constexpr (SH::WIDE) {
+                    *reinterpret_cast<uint32_t*>(col + m * 256) = pos ? up : down;
+                    *reinterpret_cast<uint32_t*>(col + (m + NPAT) * 256) = pos ? down : up;
+                } else {
+                    *reinterpret_cast<uint16_t*>(col + m * 256) = (uint16_t)((pos ? up : down) >> 16);
+                    *reinterpret_cast<uint16_t*>(col + (m + NPAT) * 256) = (uint16_t)((pos ? down : up) >> 16);
+                }
             }
         }
     }
@@ -208,47 +225,158 @@ __device__ __noinline__ bool tab_exact(const RealInst& in, float beta, int p, in
     if (q >= SH::NH) return false;
     float J[2 * D], h;
     tab_couplings<D, L, FIELD>(in, p, q, J, h);
-    const float x = tab_rule<D>(J, h, beta, pat & ((1u << SH::KI) - 1u));
+    const float f = add32(tab_sum<2 * D>(J, pat & ((1u << SH::KI) - 1u)), h);
+    const float x = mul32(beta, mul32(f, 2.0f));
     return accept_real_exact(((pat >> SH::KI) & 1u) ? -x : x, r);
 }
 
-// energies of every site and pattern: -(sum over its +e_d bonds of J S S' ) - h S
-template <int D, int L, bool FIELD>
+// energies of every site and pattern of its +e_d bonds (and own spin), rows of 32
+// columns of type A (64 bits, in units of 2^(shift - 96), or 128)
+template <int D, int L, bool FIELD, class A>
 __device__ __forceinline__ void tab_stage_energies(const RealInst& in, unsigned char* smem)
 {
     using SH = TabShape<D, L, FIELD>;
     using LT = Lat<D, L>;
     constexpr int N = SH::N, NCOL = 2 * 4 * SH::NBLK * 32;
+    auto value = [&](const longlong2* p) -> A {
+        const longlong2 v = __ldg(p);
+        const __int128 x = ((__int128)v.y << 64) | (unsigned long long)v.x;
+        return sizeof(A) == 8 ? (A)(x >> in.eshift) : (A)x;
+    };
     for (int it = threadIdx.x; it < NCOL; it += kTabThreads) {
         const int lane = it & 31, c = it >> 5;
         const int blk = c % SH::NBLK, t = (c / SH::NBLK) & 3, p = c / (4 * SH::NBLK);
         const int q = 4 * (blk * 32 + lane % SH::SEG) + t;
         const bool valid = q < SH::NH;
-        __int128 J[D], h = 0;
+        A J[D], h = 0;
+#pragma unroll
+        for (int d = 0; d < D; ++d) J[d] = 0;
         if (valid) {
             const auto nb = LT::neighbours(p, q);
 #pragma unroll
-            for (int d = 0; d < D; ++d) {
-                const longlong2 v = __ldg(&in.Jfix[d * N + nb.site]);
-                J[d] = ((__int128)v.y << 64) | (unsigned long long)v.x;
-            }
-            if (FIELD) {
-                const longlong2 v = __ldg(&in.hfix[nb.site]);
-                h = ((__int128)v.y << 64) | (unsigned long long)v.x;
-            }
+            for (int d = 0; d < D; ++d) J[d] = value(&in.Jfix[d * N + nb.site]);
+            if (FIELD) h = value(&in.hfix[nb.site]);
         }
         for (int m = 0; m < SH::EROWS; ++m) {
-            __int128 e = 0;
-            if (valid) {
+            A e = 0;
 #pragma unroll
-                for (int d = 0; d < D; ++d) e += ((m >> d) & 1) ? J[d] : -J[d];
-                if (FIELD) e += ((m >> D) & 1) ? h : -h;
-            }
-            longlong2 o;
-            o.x = (long long)(unsigned long long)e;
-            o.y = (long long)(e >> 64);
-            *reinterpret_cast<longlong2*>(smem + ((size_t)((p * 4 + t) * SH::NBLK + blk) * SH::EROWS + m) * 512 + lane * 16) = o;
+            for (int d = 0; d < D; ++d) e += ((m >> d) & 1) ? J[d] : -J[d];
+            if (FIELD) e += ((m >> D) & 1) ? h : -h;
+            *reinterpret_cast<A*>(smem + (((size_t)((p * 4 + t) * SH::NBLK + blk) * SH::EROWS + m) * 32 + lane) * sizeof(A)) = e;
         }
+    }
+}
+
+// Energies of the block's replicas: exact sums of J 2^96 as int128, accumulated
+// as 64-bit integers where every coupling and field is a multiple of 2^shift and
+// the largest possible sum fits (in.eshift >= 0: half the additions, shuffles and
+// table bytes).
+template <int D, int L, bool FIELD, class A>
+__device__ __forceinline__ void tab_energies(const RealInst& in, int R, int r0, int ng, int ga, int gb, int gstep,
+                                             unsigned char* smem)
+{
+    using SH = TabShape<D, L, FIELD>;
+    constexpr int NQP = SH::NQP, PLANE = SH::PLANE, ROT = sizeof(A) == 16 ? 1 : 0;
+    constexpr int ROWB = 32 * (int)sizeof(A);  // bytes of a row: 256 or 512
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int slot = tid / NQP, quad = tid - slot * NQP;
+    const bool owner = quad < SH::NQ;
+    const uint32_t* spin = reinterpret_cast<const uint32_t*>(smem + SH::O_SPIN);
+    const unsigned char* planes = smem + SH::O_SPIN;
+    const uint4* offs = reinterpret_cast<const uint4*>(smem + SH::O_OFFS);
+    tab_stage_energies<D, L, FIELD, A>(in, smem);
+    __syncthreads();
+    auto store = [&](int r, A v) {
+        const __int128 x = sizeof(A) == 8 ? (__int128)v << in.eshift : (__int128)v;
+        longlong2 o;
+        o.x = (long long)(unsigned long long)x;
+        o.y = (long long)(x >> 64);
+        in.E[r] = o;
+    };
+    auto shfl = [](const A& v, int off) -> A {
+        if constexpr (sizeof(A) == 8) return __shfl_xor_sync(0xffffffffu, v, off);
+        else {
+            const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)v, off);
+            const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(v >> 64), off);
+            return (A)(((unsigned __int128)hi << 64) | lo);
+        }
+    };
+    A* part = reinterpret_cast<A*>(smem + SH::O_EPART);
+    const int wsl = quad >> 5;  // this warp's index within its slot
+    const int gn = NQP < 32 ? (ng + SH::SLOTS - 1) / SH::SLOTS : gb - ga;  // warp-uniform trip count
+    const uint32_t ecol = (uint32_t)((quad >> 5) * SH::EROWS * ROWB + lane * (int)sizeof(A));
+    const uint32_t ehi = ((ecol >> 8) & 0xFFu) * 0x01010101u;
+    int wheld = -1;
+    uint32_t u[8][D + FIELD];  // pattern bits of the thread's eight sites, bit d rotated left by d + ROT
+    for (int n = 0; n < gn; ++n) {
+        const int g = ga + n * gstep;
+        const bool act = g < gb;
+        A e[4] = {0, 0, 0, 0};
+        if (act && owner) {
+            const int w = g >> 3, j = g & 7;
+            if (w != wheld) {
+                wheld = w;
+#pragma unroll
+                for (int pt = 0; pt < 8; ++pt) {
+                    const uint4 o = offs[pt * NQP + quad];
+                    const uint32_t op[3] = {o.x >> 16, o.y >> 16, o.z >> 16};
+                    const uint32_t own = spin[w * PLANE + pt * NQP + quad];
+                    const unsigned char* oth = planes + (w * PLANE + ((pt >> 2) ^ 1) * 4 * NQP) * 4;
+#pragma unroll
+                    for (int dd = 0; dd < D; ++dd)
+                        u[pt][dd] = rotl32(own ^ *reinterpret_cast<const uint32_t*>(oth + op[dd]), dd + ROT);
+                    if (FIELD) u[pt][D] = rotl32(own, D + ROT);
+                }
+            }
+            const uint32_t bit = rotl32(0x01010101u, j + ROT);
+#pragma unroll
+            for (int pt = 0; pt < 8; ++pt) {
+                // the pattern (twice the pattern for rows of 512 bytes) in each byte
+                uint32_t x = 0;
+#pragma unroll
+                for (int dd = 0; dd < D + FIELD; ++dd) x |= u[pt][dd] & rotl32(bit, dd);
+                x = rotr32(x, j) | ehi;
+                const unsigned char* et = smem + (size_t)pt * SH::NBLK * SH::EROWS * ROWB;
+                e[0] += *reinterpret_cast<const A*>(et + tab_addr<0>(x, ecol));
+                e[1] += *reinterpret_cast<const A*>(et + tab_addr<1>(x, ecol));
+                e[2] += *reinterpret_cast<const A*>(et + tab_addr<2>(x, ecol));
+                e[3] += *reinterpret_cast<const A*>(et + tab_addr<3>(x, ecol));
+            }
+        }
+        // sum over the quads; the first two steps also halve the replicas a
+        // lane holds (lane bits 0 and 1 of the slot: replica)
+        auto put = [&](int b, const A& v) {
+            if constexpr (SH::NBLK > 1) part[(g * SH::NBLK + wsl) * 4 + b] = v;
+            else if (r0 + 4 * g + b < R) store(r0 + 4 * g + b, v);
+        };
+        if constexpr (SH::SEG >= 4) {
+            const bool h0 = lane & 1, h1 = lane & 2;
+            A k0 = (h0 ? e[1] : e[0]) + shfl(h0 ? e[0] : e[1], 1);
+            A k1 = (h0 ? e[3] : e[2]) + shfl(h0 ? e[2] : e[3], 1);
+            A k = (h1 ? k1 : k0) + shfl(h1 ? k0 : k1, 2);
+#pragma unroll
+            for (int off = 4; off < SH::SEG; off <<= 1) k += shfl(k, off);
+            if (act && (lane & (SH::SEG - 1)) < 4) put(lane & 3, k);
+        } else {
+#pragma unroll
+            for (int off = 1; off < SH::SEG; off <<= 1) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) e[b] += shfl(e[b], off);
+            }
+            if (act && (lane & (SH::SEG - 1)) == 0) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) put(b, e[b]);
+            }
+        }
+    }
+    __syncthreads();  // the table, the planes and the parts are reused by the next chunk
+    if constexpr (SH::NBLK > 1) {
+        for (int t = tid; t < 4 * ng; t += kTabThreads) {
+            A e = 0;
+            for (int k = 0; k < SH::NBLK; ++k) e += part[((t >> 2) * SH::NBLK + k) * 4 + (t & 3)];
+            if (r0 + t < R) store(r0 + t, e);
+        }
+        __syncthreads();
     }
 }
 
@@ -276,44 +404,46 @@ __device__ __forceinline__ void sweep_real_table(const RealStep& s, const RealIn
     const uint4* offs = reinterpret_cast<const uint4*>(smem + SH::O_OFFS);
     unsigned char* planes = smem + SH::O_SPIN;
     const uint16_t* pos = reinterpret_cast<const uint16_t*>(smem + SH::O_POS);
-    const int nchunk = in.NP / 16;
+    constexpr int NC = (N + 31) / 32;
     const int lr = 4 * (lane & 7) + (lane >> 3);  // the replica of this lane's bit within its plane
 
-    // ---- rows (gathered through parent) -> planes: one ballot per site.  The
-    // parents go to shared memory first, and a warp has eight row pieces in
-    // flight (one at a time, two dependent loads each, took a quarter of the
-    // kernel at 3D L = 10 with 132 replicas a block)
+    // ---- rows (gathered through parent) -> planes, 32 sites at a time: a lane
+    // packs the sign bits of its replica, a transpose across the warp gives it a
+    // site's word.  The parents go to shared memory first, and a warp has four
+    // row pieces in flight (one at a time, two dependent loads each, took a
+    // quarter of the kernel at 3D L = 10 with 132 replicas a block)
     int* psrc = reinterpret_cast<int*>(smem + SH::O_SRC);
     for (int t = tid; t < 32 * nw; t += kTabThreads) {
         const int r = r0 + t;
         psrc[t] = r < R && t < 4 * ng ? (in.parent ? in.parent[r] : r) : -1;
     }
     __syncthreads();  // offsets, positions, parents are staged
-    constexpr int kBatch = 8;
-    for (int tup0 = warp; tup0 < nw * nchunk; tup0 += NWARP * kBatch) {
-        uint4 v[kBatch];
+    constexpr int kBatch = 4;
+    for (int tup0 = warp; tup0 < nw * NC; tup0 += NWARP * kBatch) {
+        uint4 v[kBatch][2];
 #pragma unroll
         for (int x = 0; x < kBatch; ++x) {
-            const int tup = tup0 + x * NWARP, w = tup / nchunk, c = tup - w * nchunk;
-            v[x] = make_uint4(0u, 0u, 0u, 0u);
-            if (tup < nw * nchunk) {
-                const int src = psrc[32 * w + lr];
-                if (src >= 0) v[x] = *reinterpret_cast<const uint4*>(in.Sin + (size_t)src * in.NP + 16 * c);
+            const int tup = tup0 + x * NWARP, w = tup / NC, c = tup - w * NC;
+            v[x][0] = v[x][1] = make_uint4(0u, 0u, 0u, 0u);
+            const int src = tup < nw * NC ? psrc[32 * w + lr] : -1;
+            if (src >= 0) {
+                const uint4* row = reinterpret_cast<const uint4*>(in.Sin + (size_t)src * in.NP + 32 * c);
+                v[x][0] = row[0];
+                if (32 * c + 16 < in.NP) v[x][1] = row[1];
             }
         }
 #pragma unroll
         for (int x = 0; x < kBatch; ++x) {
-            const int tup = tup0 + x * NWARP, w = tup / nchunk, c = tup - w * nchunk;
-            if (tup >= nw * nchunk) break;  // warp-uniform
-            const uint32_t wv[4] = {v[x].x, v[x].y, v[x].z, v[x].w};
-            uint32_t mine = 0;
+            const int tup = tup0 + x * NWARP, w = tup / NC, c = tup - w * NC;
+            if (tup >= nw * NC) break;  // warp-uniform
+            const uint32_t wv[8] = {v[x][0].x, v[x][0].y, v[x][0].z, v[x][0].w, v[x][1].x, v[x][1].y, v[x][1].z, v[x][1].w};
+            uint32_t bits = 0;
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
-                const uint32_t bal = __ballot_sync(0xffffffffu, (wv[t >> 2] >> (8 * (t & 3) + 7)) & 1u);
-                if (lane == t) mine = bal;
-            }
-            const int i = 16 * c + lane;
-            if (lane < 16 && i < N) *reinterpret_cast<uint32_t*>(planes + w * PLANE * 4 + pos[i]) = mine;
+            for (int t = 0; t < 8; ++t)  // bit 7 of the four bytes, gathered by a multiply
+                bits |= ((((wv[t] >> 7) & 0x01010101u) * 0x01020408u) >> 24) << (4 * t);
+            const uint32_t mine = transpose32(bits, lane);
+            const int i = 32 * c + lane;
+            if (i < N) *reinterpret_cast<uint32_t*>(planes + w * PLANE * 4 + pos[i]) = mine;
         }
     }
     if constexpr (NH % 4 != 0) {  // the last quad's missing sites
@@ -476,128 +606,25 @@ __device__ __forceinline__ void sweep_real_table(const RealStep& s, const RealIn
             for (int dd = 0; dd < D; ++dd) gJ[dd * N + i] += nrep - 2 * diff[dd];
         }
     }
-    // ---- rows out
-    for (int tup = warp; tup < nw * nchunk; tup += NWARP) {
-        const int w = tup / nchunk, c = tup - w * nchunk;
-        uint32_t wv[4];
+    // ---- rows out: the transpose back, then a byte per bit
+    for (int tup = warp; tup < nw * NC; tup += NWARP) {
+        const int w = tup / NC, c = tup - w * NC, i = 32 * c + lane;
+        const uint32_t bits =
+            transpose32(i < N ? *reinterpret_cast<const uint32_t*>(planes + w * PLANE * 4 + pos[i]) : 0u, lane);
+        uint32_t wv[8];
 #pragma unroll
-        for (int t4 = 0; t4 < 4; ++t4) {
-            uint32_t x = 0;
-            if (16 * c + 4 * t4 < N) {
-                const uint2 o = *reinterpret_cast<const uint2*>(pos + 16 * c + 4 * t4);
-                const unsigned char* pl = planes + w * PLANE * 4;
-                const uint32_t o4[4] = {o.x & 0xFFFFu, o.x >> 16, o.y & 0xFFFFu, o.y >> 16};
-#pragma unroll
-                for (int t = 0; t < 4; ++t) x |= ((*reinterpret_cast<const uint32_t*>(pl + o4[t]) >> lane) & 1u) << (8 * t);
-            }
-            wv[t4] = (x * 0xFEu) ^ 0x01010101u;  // 1 -> -1 (0xFF), 0 -> +1
-        }
+        for (int t = 0; t < 8; ++t)  // 1 -> -1 (0xFF), 0 -> +1
+            wv[t] = (((((bits >> (4 * t)) & 15u) * 0x00204081u) & 0x01010101u) * 0xFEu) ^ 0x01010101u;
         const int r = r0 + 32 * w + lr;
-        if (r < R && 32 * w + lr < 4 * ng)
-            *reinterpret_cast<uint4*>(in.Sout + (size_t)r * in.NP + 16 * c) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-    }
-    // ---- energies (exact, int128): the table gives way to the sites' energies
-    tab_stage_energies<D, L, FIELD>(in, smem);
-    __syncthreads();
-    longlong2* part = reinterpret_cast<longlong2*>(smem + SH::O_EPART);
-    const int wsl = (quad >> 5);  // this warp's index within its slot
-    const int gn = NQP < 32 ? (ng + SH::SLOTS - 1) / SH::SLOTS : gb - ga;  // warp-uniform trip count
-    const uint32_t ecol = (uint32_t)((quad >> 5) * SH::EROWS * 512 + lane * 16);
-    const uint32_t ehi = ((ecol >> 8) & 0xFFu) * 0x01010101u;
-    int wheld = -1;
-    uint32_t u[8][D + FIELD];  // pattern bits of the thread's eight sites, bit d rotated left by d + 1
-    for (int n = 0; n < gn; ++n) {
-        const int g = ga + n * gstep;
-        const bool act = g < gb;
-        unsigned __int128 e[4] = {0, 0, 0, 0};
-        if (act && owner) {
-            const int w = g >> 3, j = g & 7;
-            if (w != wheld) {
-                wheld = w;
-#pragma unroll
-                for (int pt = 0; pt < 8; ++pt) {
-                    const uint4 o = offs[pt * NQP + quad];
-                    const uint32_t op[3] = {o.x >> 16, o.y >> 16, o.z >> 16};
-                    const uint32_t own = spin[w * PLANE + pt * NQP + quad];
-                    const unsigned char* oth = planes + (w * PLANE + ((pt >> 2) ^ 1) * 4 * NQP) * 4;
-#pragma unroll
-                    for (int dd = 0; dd < D; ++dd)
-                        u[pt][dd] = rotl32(own ^ *reinterpret_cast<const uint32_t*>(oth + op[dd]), dd + 1);
-                    if (FIELD) u[pt][D] = rotl32(own, D + 1);
-                }
-            }
-            const uint32_t bit = rotl32(0x01010101u, j);
-#pragma unroll
-            for (int pt = 0; pt < 8; ++pt) {
-                // twice the pattern in each byte: rows of 512 bytes
-                uint32_t x = 0;
-#pragma unroll
-                for (int dd = 0; dd < D + FIELD; ++dd) x |= u[pt][dd] & rotl32(bit, dd + 1);
-                x = rotr32(x, j) | ehi;
-                const unsigned char* et = smem + (size_t)pt * SH::NBLK * SH::EROWS * 512;
-                auto add = [&](auto BB) {
-                    constexpr int b = decltype(BB)::value;
-                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(
-                        et + tab_addr<b>(x, ecol));
-                    e[b] += ((unsigned __int128)v.y << 64) | v.x;
-                };
-                add(std::integral_constant<int, 0>{});
-                add(std::integral_constant<int, 1>{});
-                add(std::integral_constant<int, 2>{});
-                add(std::integral_constant<int, 3>{});
-            }
-        }
-        // sum over the quads; the first two steps also halve the replicas a
-        // lane holds (lane bits 0 and 1 of the slot: replica)
-        auto add_from = [](unsigned __int128& x, const unsigned __int128& give, int off) {
-            const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)give, off);
-            const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(give >> 64), off);
-            x += ((unsigned __int128)hi << 64) | lo;
-        };
-        auto put = [&](int b, const unsigned __int128& v) {
-            longlong2 o;
-            o.x = (long long)(unsigned long long)v;
-            o.y = (long long)(unsigned long long)(v >> 64);
-            if constexpr (SH::NBLK > 1) part[(g * SH::NBLK + wsl) * 4 + b] = o;
-            else if (r0 + 4 * g + b < R) in.E[r0 + 4 * g + b] = o;
-        };
-        if constexpr (SH::SEG >= 4) {
-            const bool h0 = lane & 1, h1 = lane & 2;
-            unsigned __int128 k0 = h0 ? e[1] : e[0], k1 = h0 ? e[3] : e[2];
-            add_from(k0, h0 ? e[0] : e[1], 1);
-            add_from(k1, h0 ? e[2] : e[3], 1);
-            unsigned __int128 k = h1 ? k1 : k0;
-            add_from(k, h1 ? k0 : k1, 2);
-#pragma unroll
-            for (int off = 4; off < SH::SEG; off <<= 1) add_from(k, k, off);
-            if (act && (lane & (SH::SEG - 1)) < 4) put(lane & 3, k);
-        } else {
-#pragma unroll
-            for (int off = 1; off < SH::SEG; off <<= 1) {
-#pragma unroll
-                for (int b = 0; b < 4; ++b) add_from(e[b], e[b], off);
-            }
-            if (act && (lane & (SH::SEG - 1)) == 0) {
-#pragma unroll
-                for (int b = 0; b < 4; ++b) put(b, e[b]);
-            }
+        if (r < R && 32 * w + lr < 4 * ng) {
+            uint4* row = reinterpret_cast<uint4*>(in.Sout + (size_t)r * in.NP + 32 * c);
+            row[0] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+            if (32 * c + 16 < in.NP) row[1] = make_uint4(wv[4], wv[5], wv[6], wv[7]);
         }
     }
-    __syncthreads();  // the table, the planes and the parts are reused by the next chunk
-    if constexpr (SH::NBLK > 1) {
-        for (int t = tid; t < 4 * ng; t += kTabThreads) {
-            unsigned __int128 e = 0;
-            for (int k = 0; k < SH::NBLK; ++k) {
-                const longlong2 v = part[((t >> 2) * SH::NBLK + k) * 4 + (t & 3)];
-                e += ((unsigned __int128)(unsigned long long)v.y << 64) | (unsigned long long)v.x;
-            }
-            longlong2 o;
-            o.x = (long long)(unsigned long long)e;
-            o.y = (long long)(unsigned long long)(e >> 64);
-            if (r0 + t < R) in.E[r0 + t] = o;
-        }
-        __syncthreads();
-    }
+    // ---- energies: the table gives way to the sites' energies
+    if (in.eshift >= 0) tab_energies<D, L, FIELD, long long>(in, R, r0, ng, ga, gb, gstep, smem);
+    else tab_energies<D, L, FIELD, __int128>(in, R, r0, ng, ga, gb, gstep, smem);
 }
 
 // zero the block's gradient sums; add them to the step's counters at the end
