@@ -199,6 +199,14 @@ struct ResampleArgs {
     int32_t* bcount;             // [rs_scan_blocks] copies per scan block
     int32_t* blocksum;           // a shard: scratch for the count scan
     double* lnQ_out;             // ln Q once more (or null)
+    int self;                    // 1 (one-launch populations only): take E_min from E32 (and write it to
+                                 // prev) and zero the copy numbers first
+    int32_t* parent;             // [R] out
+    const int32_t* fam_in;       // [R]
+    int32_t* fam_out;            // [R]
+    double dbeta, log_R, betaF0;
+    int k;
+    uint32_t key0, key1, c3;
 };
 // Weight prefix in a fixed order of fan-out kFan: runs of kFan weights summed
 // left to right, the run totals likewise, recursively; each weights block
@@ -231,6 +239,7 @@ __host__ __device__ constexpr inline int rs_bcount_size(int R)
 }
 cudaError_t launch_resample(const ResampleArgs& a, cudaStream_t st);
 int resample_launches(const ResampleArgs& a);  // kernels that launch_resample enqueues
+bool resample_one_launch(int R);
 // one phase (0..3) of a shard's resampling (a.gR > 0, a.sync null)
 cudaError_t launch_resample_shard(const ResampleArgs& a, int phase, cudaStream_t st);
 // all instances of a batch at once: tab[i] describes instance i (device memory)

@@ -31,9 +31,7 @@ constexpr int kMaxUpper = 2 * ((kMaxR + pa::kWBlock - 1) / pa::kWBlock) + 64;  /
 constexpr size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t kOffP = 0;
 constexpr size_t kOffCounts = kOffP + al(sizeof(double) * kMaxR);
-constexpr size_t kOffFamIn = kOffCounts + al(sizeof(int32_t) * kMaxR);
-constexpr size_t kOffFamOut = kOffFamIn + al(sizeof(int32_t) * kMaxR);
-constexpr size_t kOffLev1 = kOffFamOut + al(sizeof(int32_t) * kMaxR);
+constexpr size_t kOffLev1 = kOffCounts + al(sizeof(int32_t) * kMaxR);
 constexpr size_t kOffBmax = kOffLev1 + al(sizeof(double) * kMaxLeaves);
 constexpr size_t kOffUpper = kOffBmax + al(sizeof(double) * 2 * ((kMaxR + pa::kWBlock - 1) / pa::kWBlock));
 constexpr size_t kOffRunP = kOffUpper + al(sizeof(double) * kMaxUpper);
@@ -57,18 +55,16 @@ std::mutex g_mu;
 unsigned char* g_addr[kMaxDevices] = {};
 
 // E_min into prev (as pa_anneal_step takes it from the previous step's
-// observables), zero copy counts, identity families, zero running sums.
+// observables), zero copy counts, zero running sums.
 __global__ void __launch_bounds__(1024) static_prep_kernel(const int32_t* E, int R, unsigned char* base)
 {
     __shared__ int wmin[32];
     int32_t* counts = reinterpret_cast<int32_t*>(base + kOffCounts);
-    int32_t* fam = reinterpret_cast<int32_t*>(base + kOffFamIn);
     pa::StepAcc* acc = reinterpret_cast<pa::StepAcc*>(base + kOffAcc);
     int mn = 0x7fffffff;
     for (int r = threadIdx.x; r < R; r += blockDim.x) {
         mn = min(mn, E[r]);
         counts[r] = 0;
-        fam[r] = r;
     }
     mn = __reduce_min_sync(0xffffffffu, mn);
     if ((threadIdx.x & 31) == 0) wmin[threadIdx.x >> 5] = mn;
@@ -130,8 +126,9 @@ extern "C" int pa_resample_static(const int32_t* d_E, int R, double beta_prev, d
         base = g_addr[dev];
     }
     cudaStream_t st = (cudaStream_t)stream;
-    static_prep_kernel<<<1, 1024, 0, st>>>(d_E, R, base);
     pa::ResampleArgs ra{};
+    ra.self = pa::resample_one_launch(R) ? 1 : 0;
+    if (!ra.self) static_prep_kernel<<<1, 1024, 0, st>>>(d_E, R, base);
     ra.R = R;
     ra.Rn = R;
     ra.kind = 0;
@@ -150,8 +147,6 @@ extern "C" int pa_resample_static(const int32_t* d_E, int R, double beta_prev, d
     ra.sync = reinterpret_cast<int*>(base + kOffSync);
     ra.lnQ_out = d_lnQ;
     ra.parent = d_parent;
-    ra.fam_in = reinterpret_cast<const int32_t*>(base + kOffFamIn);
-    ra.fam_out = reinterpret_cast<int32_t*>(base + kOffFamOut);
     ra.dbeta = beta_next - beta_prev;
     ra.log_R = std::log((double)R);
     ra.betaF0 = 0.0;

@@ -74,7 +74,7 @@ __device__ __forceinline__ int rs_src(const ResampleArgs& a) { return a.Rsrc ? *
 // finalize 24 us -> 16 us, most of it 62-cycle FP64 additions in a chain.
 constexpr int kFuseR = 128 * kWBlock;
 template <int T>
-__device__ __forceinline__ void rs_levels_body(const ResampleArgs& a, int b, int R)
+__device__ __forceinline__ void rs_levels_body(const ResampleArgs& a, int b, int R, int emin)
 {
     constexpr int PER = kWBlock / T;
     __shared__ double s_w[kFan * (kFan + 1)];  // run c at [c (kFan + 1)], padded against bank conflicts
@@ -85,7 +85,6 @@ __device__ __forceinline__ void rs_levels_body(const ResampleArgs& a, int b, int
     const int n = min(kWBlock, R - i0);
     if (tid == 0 && a.bcount && b < rs_scan_blocks(R)) a.bcount[b] = 0;
     if (a.kind == 0) {
-        const int emin = (int)a.prev->emin_lo;
         int lv[PER], lo = 0x7fffffff, hi = -1;
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
@@ -259,7 +258,7 @@ __device__ __forceinline__ void rs_weights_launch(const ResampleArgs& a, int b)
 {
     const int R = rs_src(a), live = rs_live_blocks(R);
     if (b >= live) return;  // block-uniform: past the source population
-    rs_levels_body<T>(a, b, R);
+    rs_levels_body<T>(a, b, R, (int)a.prev->emin_lo);
     if (!last_block(a.sync, live)) return;
     if (T == kWBlock) rs_fused(a, R);
     else rs_top_body(a);  // levels >= 2 of the prefix
@@ -273,7 +272,7 @@ __global__ void __launch_bounds__(kWThreads) rs_weights_batched(const ResampleAr
 // a shard: the levels >= 2 need every shard's block totals
 __global__ void __launch_bounds__(kWThreads) rs_weights_shard_kernel(ResampleArgs a)
 {
-    rs_levels_body<kWThreads>(a, blockIdx.x, a.R);
+    rs_levels_body<kWThreads>(a, blockIdx.x, a.R, (int)a.prev->emin_lo);
 }
 
 // Levels >= 2 of the prefix, by one block: bottom-up sums inside runs of the nb
@@ -616,6 +615,14 @@ __global__ void __launch_bounds__(kDrawThreads) rs_draws_batched(const ResampleA
 // nearest-integer copy numbers (Sec. II.B, population in expectation):
 // tau_i = target w_i / S, n_i = floor(tau_i) + [u_i < tau_i - floor(tau_i)],
 // u_i from the RESAMPLE stream at counter (i, k, 1)
+__device__ __forceinline__ int rs_nearest_copies(const ResampleArgs& a, int i, double S)
+{
+    const u32x4 o = philox((uint32_t)i, (uint32_t)a.k, 1u, a.c3, a.key0, a.key1);
+    const double u = uniform53(o.x, o.y);
+    const double tau = __ddiv_rn(__dmul_rn(a.target, a.w[i]), S);
+    const double fl = floor(tau);
+    return (int32_t)fl + (u < __dsub_rn(tau, fl) ? 1 : 0);
+}
 __global__ void __launch_bounds__(256) rs_nearest_kernel(ResampleArgs a)
 {
     __shared__ int s_n[8];
@@ -623,12 +630,7 @@ __global__ void __launch_bounds__(256) rs_nearest_kernel(ResampleArgs a)
     if ((int)blockIdx.x * 256 >= R) return;  // block-uniform
     int n = 0;
     if (i < R) {
-        const double S = a.cur->S;
-        const u32x4 o = philox((uint32_t)i, (uint32_t)a.k, 1u, a.c3, a.key0, a.key1);
-        const double u = uniform53(o.x, o.y);
-        const double tau = __ddiv_rn(__dmul_rn(a.target, a.w[i]), S);
-        const double fl = floor(tau);
-        n = (int32_t)fl + (u < __dsub_rn(tau, fl) ? 1 : 0);
+        n = rs_nearest_copies(a, i, a.cur->S);
         a.counts[i] = n;
     }
     n = __reduce_add_sync(0xffffffffu, n);
@@ -753,13 +755,13 @@ __device__ __forceinline__ void rs_place_body(const ResampleArgs& a, int b, int 
 #pragma unroll
     for (int t = 0; t < PER; ++t) {
         const int i = i0 + tid * PER + t;
-        c[t] = i < R ? a.counts[i] : 0;
-        s_fam[tid * PER + t] = i < R ? a.fam_in[i] : 0;
+        c[t] = i < R ? __ldcg(a.counts + i) : 0;
+        s_fam[tid * PER + t] = i < R && a.fam_in ? a.fam_in[i] : 0;
         s += c[t];
         c[t] = s;
     }
     for (int t = tid; t < ((a.Rdst && b == 0) ? ns : b); t += 1024) {
-        const int v = a.bcount[t];
+        const int v = __ldcg(a.bcount + t);
         all += v;
         if (t < b) pre += v;
     }
@@ -799,9 +801,114 @@ __device__ __forceinline__ void rs_place_body(const ResampleArgs& a, int b, int 
             if (t < s_cum[mid]) hi = mid; else lo = mid + 1;
         }
         a.parent[off + t] = i0 + lo;
-        a.fam_out[off + t] = s_fam[lo];
+        if (a.fam_out) a.fam_out[off + t] = s_fam[lo];
     }
 }
+
+// A population of at most kClusterR replicas: the whole resampling in one launch
+// of one cluster, a CTA per weights block.  The steps between which the larger
+// populations change launches are cluster barriers here (every CTA of a cluster
+// is resident, and the barrier's release and acquire order the global writes),
+// and every CTA completes the few values above its block by itself.  R = 1000:
+// 25 -> XX us.
+constexpr int kClusterCtas = 8;  // the portable cluster size
+constexpr int kClusterR = kClusterCtas * kWBlock;
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__global__ void __launch_bounds__(kWBlock) rs_cluster_kernel(ResampleArgs a)
+{
+    constexpr int kRuns = kClusterCtas * kFan;
+    __shared__ double s_up[kClusterCtas], s_rp[kRuns], s_rq[kRuns];
+    __shared__ long long s_end[kClusterCtas];
+    __shared__ int s_hist[kClusterCtas], s_min[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b = blockIdx.x, R = rs_src(a), nb = rs_wblocks(R), leaves = rs_leaves(R);
+    int emin = 0;
+    if (a.self) {
+        // no earlier launch: E_min, and the copy numbers' initial zeros
+        int m = 0x7fffffff;
+        for (int t = tid; t < R; t += kWBlock) m = min(m, a.E32[t]);
+        m = __reduce_min_sync(0xffffffffu, m);
+        if (lane == 0) s_min[warp] = m;
+        __syncthreads();
+        emin = __reduce_min_sync(0xffffffffu, s_min[lane]);
+        if (b * kWBlock + tid < R) a.counts[b * kWBlock + tid] = 0;
+        if (b == 0 && tid == 0) {
+            StepAcc* prev = const_cast<StepAcc*>(a.prev);
+            prev->emin_lo = emin;
+            prev->emin_hi = emin < 0 ? -1 : 0;
+            prev->sum_lnQ = 0.0;
+        }
+    } else if (a.kind == 0) {
+        emin = (int)a.prev->emin_lo;
+    }
+    if (b < rs_live_blocks(R)) rs_levels_body<kWBlock>(a, b, R, emin);
+    cluster_sync();
+    if (tid == 0) {  // at most kFan block totals: one run of the next level
+        double acc = 0.0;
+        for (int t = 0; t < nb; ++t) {
+            const double v = __ldcg(a.upper + t);
+            acc = t == 0 ? v : __dadd_rn(acc, v);
+            s_up[t] = acc;
+        }
+    }
+    if (tid < kClusterCtas) s_hist[tid] = 0;
+    __syncthreads();
+    if (warp == 0 && b < nb) {
+        const long long m = rs_run_table(a, b, R, s_up);
+        if (lane == 0) a.bmax[b] = __longlong_as_double(m);
+    }
+    cluster_sync();
+    for (int t = tid; t < leaves; t += kWBlock) {
+        s_rp[t] = __ldcg(a.runP + t);
+        s_rq[t] = __ldcg(a.runq + t);
+    }
+    if (tid == 0) {
+        long long m = 0;
+        for (int t = 0; t < nb; ++t) {
+            m = max(m, dbits(__ldcg(a.bmax + t)));
+            s_end[t] = m;
+        }
+        if (b == 0) a.cur->S = __longlong_as_double(m);
+    }
+    __syncthreads();
+    const double S = nb > 0 ? __longlong_as_double(s_end[nb - 1]) : 0.0;
+    if (a.scheme == 1) {
+        const int i = b * kWBlock + tid;
+        int n = 0;
+        if (i < R) {
+            n = rs_nearest_copies(a, i, S);
+            a.counts[i] = n;
+        }
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (lane == 0 && n) atomicAdd(&s_hist[b], n);
+    } else {
+        for (int q = b * kWBlock + tid; q < a.Rn; q += gridDim.x * kWBlock) {
+            const u32x4 o = philox((uint32_t)q, (uint32_t)a.k, 0u, a.c3, a.key0, a.key1);
+            const long long x = dbits(__dmul_rn(uniform53(o.x, o.y), S));  // x >= 0
+            const bool strict = x < s_end[nb - 1];  // else x == S after rounding: the first P >= x
+            auto past = [&](long long p) { return strict ? x < p : p >= x; };
+            int bl = 0;
+            while (bl < nb - 1 && !past(s_end[bl])) ++bl;
+            const int c = min(leaves - 1, bl * kFan + first_of_32([&](int t) {
+                return bl * kFan + t >= leaves || past(dbits(s_rp[bl * kFan + t]));
+            }));
+            const double qc = s_rq[c];
+            const int i = min(R - 1, c * kFan + first_of_32([&](int t) {
+                return c * kFan + t >= R || past(dbits(__dadd_rn(qc, __ldcg(a.P + c * kFan + t))));
+            }));
+            atomicAdd(&a.counts[i], 1);
+            atomicAdd(&s_hist[i / kWBlock], 1);
+        }
+    }
+    __syncthreads();
+    if (tid < nb && s_hist[tid]) atomicAdd(&a.bcount[tid], s_hist[tid]);
+    cluster_sync();
+    if (b < max(1, rs_scan_blocks(R))) rs_place_body<kWBlock>(a, b, R);
+}
+
 __device__ __forceinline__ void rs_place_launch(const ResampleArgs& a, int b)
 {
     const int R = rs_src(a);
@@ -819,6 +926,21 @@ static int place_grid(int R) { return rs_bcount_size(R); }
 cudaError_t launch_resample(const ResampleArgs& a, cudaStream_t st)
 {
     // a.R sizes the grids (the capacity when the population is in device memory)
+    if (a.R <= kClusterR) {
+        int ctas = 1;
+        while (ctas < rs_wblocks(a.R)) ctas *= 2;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = ctas;
+        cfg.blockDim = kWBlock;
+        cfg.stream = st;
+        cudaLaunchAttribute at = {};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = ctas;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, rs_cluster_kernel, a);
+    }
     const bool fused = a.R <= kFuseR;
     if (fused) {
         rs_weights_fused_kernel<<<rs_wblocks(a.R), kWBlock, 0, st>>>(a);
@@ -835,7 +957,8 @@ cudaError_t launch_resample(const ResampleArgs& a, cudaStream_t st)
     rs_place_kernel<<<place_grid(a.R), 1024, 0, st>>>(a);
     return cudaGetLastError();
 }
-int resample_launches(const ResampleArgs& a) { return a.R <= kFuseR ? 3 : 4; }
+int resample_launches(const ResampleArgs& a) { return a.R <= kClusterR ? 1 : a.R <= kFuseR ? 3 : 4; }
+bool resample_one_launch(int R) { return R <= kClusterR; }
 
 // the phases of a shard's resampling (the host exchanges the block totals,
 // the block maxima and the copy totals between them)

@@ -5,7 +5,8 @@
   block, more levels than a block looks up, energies not congruent modulo 4, one
   replica that takes nearly every slot, equal energies.  Parents bit-exact
   against the oracle; ln Q to 1e-12 as in test_gpu_parity.
-* Populations around the largest that one launch completes (131072), above it,
+* Populations around the largest that one cluster resamples (8192: also the static
+  call), the largest whose weights launch completes the prefix (131072), above it,
   and above 2048 weights blocks (segments of two): one step of a 2D L = 2
   population against the oracle's resampling of the downloaded energies, and
   the observables against integer sums and family counts of the downloads.
@@ -35,7 +36,7 @@ def _energies(how, R, rng):
     return np.full(R, -96)
 
 
-@pytest.mark.parametrize("R", [1, 2, 31, 32, 33, 1023, 1024, 1025, 4097, 32769, 65535, 65536])
+@pytest.mark.parametrize("R", [1, 2, 31, 32, 33, 1023, 1024, 1025, 2049, 4097, 8191, 8192, 8193, 32769, 65535, 65536])
 @pytest.mark.parametrize("how", ["levels", "wide", "odd", "one", "equal"])
 def test_static_resample_edges(pa, oracle, R, how):
     import torch
@@ -50,7 +51,7 @@ def test_static_resample_edges(pa, oracle, R, how):
     assert lnq.item() == pytest.approx(want["lnQ"], rel=1e-12, abs=1e-13)
 
 
-@pytest.mark.parametrize("R", [131071, 131072, 131073, 400_001, 2_098_177])
+@pytest.mark.parametrize("R", [1025, 8192, 8193, 131071, 131072, 131073, 400_001, 2_098_177])
 def test_population_resample_sizes(pa, oracle, R):
     P, O = pa, oracle
     J, betas, seed = W.couplings_pm(2, 2, 5), np.array([0.0, 0.4, 1.1]), 99 + R
