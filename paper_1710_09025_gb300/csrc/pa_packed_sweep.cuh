@@ -22,6 +22,37 @@ __global__ void __launch_bounds__(THREADS, 4) sweep_packed_kernel(PackedSweepArg
     sweep_packed_tile<D, L, GPB, THREADS, I8, true, SHARD>(a.s, a.i, g0, gend, smem_packed);
 }
 
+// threads per word of the team variant: at most eight, at most 512 threads a
+// block; 1 where the lattice has more than 256 words per sublattice
+template <int D, int L> __host__ __device__ constexpr int team_of()
+{
+    constexpr int NH = Lat<D, L>::NH;
+    int t = 8;
+    while (t > 1 && t * NH > 512) t /= 2;
+    return t;
+}
+template <int D, int L> __host__ __device__ constexpr int team_threads()
+{
+    int n = 32;
+    while (n < team_of<D, L>() * Lat<D, L>::NH) n *= 2;
+    return n;
+}
+template <int D, int L, bool I8>
+__global__ void __launch_bounds__(team_threads<D, L>()) sweep_packed_team_kernel(PackedSweepArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem_packed[];
+    const int G = packed_groups(a.i), g0 = blockIdx.x;
+    sweep_packed_tile<D, L, 1, team_threads<D, L>(), I8, true, false, team_of<D, L>()>(a.s, a.i, g0, min(g0 + 1, G), smem_packed);
+}
+template <int D, int L, bool I8>
+static cudaError_t launch_team(const PackedSweepArgs& a, cudaStream_t st)
+{
+    constexpr size_t smem = PackedShape<D, L, 1, team_threads<D, L>(), false>::SMEM;
+    static_assert(smem <= 48 * 1024, "no opt-in needed");
+    sweep_packed_team_kernel<D, L, I8><<<a.i.G, team_threads<D, L>(), smem, st>>>(a);
+    return cudaGetLastError();
+}
+
 // ---------------- shapes and dispatch ----------------
 
 template <int D, int L, int GPB, int THREADS, bool I8, bool SHARD = false>
@@ -54,6 +85,18 @@ static cudaError_t launch_dl(const PackedSweepArgs& a, int gpb, int threads, cud
         return i8 ? launch_one<D, L, 2 * s.gpb, s.threads, true>(a, grid, 0, st)
                   : launch_one<D, L, 2 * s.gpb, s.threads, false>(a, grid, 0, st);
     if (gpb != s.gpb || threads != s.threads) return cudaErrorInvalidConfiguration;
+    // few threads to an SM even with a team per word: the team variant (us a
+    // launch before -> with it: L=4, R=1000 36 -> 18; L=4, R=30000 44 -> 38; L=6,
+    // R=5000 39 -> 29; L=8, R=5000 52 -> 36; above the line it does more work than
+    // it hides: L=6, R=30000 66 -> 86)
+    if constexpr (team_of<D, L>() > 1) {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int per_sm = team_threads<D, L>() <= 256 ? 1024 : 512;
+        if ((long long)a.i.G * team_threads<D, L>() <= (long long)sms * per_sm)
+            return i8 ? launch_team<D, L, true>(a, st) : launch_team<D, L, false>(a, st);
+    }
     // fewer than two full blocks to an SM: spread the groups over up to four
     // blocks to an SM (L=6, R=40001: 119 -> 81 us; L=6, R=5000: 116 -> 41 us;
     // 2D L=16, R=30000: 125 -> 68 us); with more full blocks than that spreading

@@ -151,12 +151,17 @@ template <int D, int L> __host__ __device__ constexpr Shape default_shape()
 // SHARD: the instance is a shard of a larger population; its PLANE counters
 // carry the global group index g0 + in.goff (a separate instantiation, so
 // that the counters of every other launch cost nothing extra)
-template <int D, int L, int GPB, int THREADS, bool I8, bool LATE = true, bool SHARD = false>
+// TEAM > 1 (one group per block): TEAM neighbouring threads share a word, for
+// populations too small to fill the GPU, where the time of one word counts and
+// not the work.  Every thread of a team classifies the word, makes one call and
+// compares its two planes; the partial results (r < thr so far, equal so far)
+// are combined in plane order across the team.
+template <int D, int L, int GPB, int THREADS, bool I8, bool LATE = true, bool SHARD = false, int TEAM = 1>
 __device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const PackedInst& in, int g0, int gend,
                                                   unsigned char* smem)
 {
     using LT = Lat<D, L>;
-    using SH = PackedShape<D, L, GPB, THREADS, LATE>;
+    using SH = PackedShape<D, L, GPB, THREADS, LATE && TEAM == 1>;
     constexpr int N = SH::N, NH = SH::NH, TPG = SH::TPG, SEGW = SH::SEGW, NSEG = SH::NSEG, B = SH::B;
     constexpr int NWARP = THREADS / 32;
     uint64_t* sm = reinterpret_cast<uint64_t*>(smem);
@@ -445,6 +450,57 @@ __device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const Pac
     // (L = 4..10, doubled groups per block) measured slower and keeps the loop
     constexpr bool kLate = SH::kLate;
 
+    if constexpr (TEAM > 1) {
+        static_assert(GPB == 1 && TEAM * NH <= THREADS && TEAM <= 16, "one group, a team per word");
+        const int q = tid / TEAM, tl = tid % TEAM;
+        const bool act = q < NH;
+        const typename LT::Nb nb0 = LT::neighbours(0, act ? q : 0), nb1 = LT::neighbours(1, act ? q : 0);
+        // threshold bits of this thread's first two planes
+        const uint32_t v00a = s.v00[2 * tl], v01a = s.v01[2 * tl], v10a = s.v10[2 * tl];
+        const uint32_t v00b = s.v00[2 * tl + 1], v01b = s.v01[2 * tl + 1], v10b = s.v10[2 * tl + 1];
+        for (int sw = 0; sw < s.n_sweeps; ++sw) {
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                const uint32_t hs = s.hs0 + 2u * (uint32_t)sw + (uint32_t)p;
+                uint64_t* cur = sm + p * NH + (act ? q : 0);
+                uint64_t b0, b1, b2, down, acc, U;
+                u32x4 o = plane_call((uint32_t)q, hs, 16u * (uint32_t)g0 + (uint32_t)tl);
+                const uint64_t sw0 = *cur;
+                count_bonds(sw0, sm + (p ^ 1) * NH, p == 0 ? nb0.q : nb1.q, sj[p * NH + (act ? q : 0)], b0, b1, b2, down);
+                start(b0, b1, b2, down, acc, U);
+                auto bit = [&](uint32_t v00, uint32_t v01, uint32_t v10) {  // the threshold bit of a lane's class
+                    const uint64_t inner = (b0 & rep32(v01)) | (~b0 & rep32(v00));
+                    return (b1 & rep32(v10)) | (~b1 & inner);
+                };
+                uint64_t T0 = bit(v00a, v01a, v10a), T1 = bit(v00b, v01b, v10b);
+#pragma unroll 1
+                for (int m = tl;;) {
+                    const uint64_t p0 = (uint64_t)o.x | ((uint64_t)o.y << 32), p1 = (uint64_t)o.z | ((uint64_t)o.w << 32);
+                    uint64_t eq = ~(T0 ^ p0);
+                    uint64_t lt = (T0 & ~p0) | (eq & T1 & ~p1);
+                    eq &= ~(T1 ^ p1);
+#pragma unroll
+                    for (int off = 1; off < TEAM; off <<= 1) {  // the next planes' results after these
+                        const uint64_t lt2 = __shfl_down_sync(0xffffffffu, lt, off, TEAM);
+                        const uint64_t eq2 = __shfl_down_sync(0xffffffffu, eq, off, TEAM);
+                        lt |= eq & lt2;
+                        eq &= eq2;
+                    }
+                    if (tl == 0) {
+                        acc |= U & lt;
+                        U &= eq;
+                    }
+                    m += TEAM;
+                    if (m >= 16 || !__any_sync(0xffffffffu, act && tl == 0 && U != 0)) break;
+                    o = plane_call((uint32_t)q, hs, 16u * (uint32_t)g0 + (uint32_t)m);
+                    T0 = bit(s.v00[2 * m], s.v01[2 * m], s.v10[2 * m]);
+                    T1 = bit(s.v00[2 * m + 1], s.v01[2 * m + 1], s.v10[2 * m + 1]);
+                }
+                if (act && tl == 0) *cur = sw0 ^ acc;
+                __syncthreads();
+            }
+        }
+    } else
     for (int sw = 0; sw < s.n_sweeps; ++sw) {
         for (int p = 0; p < 2; ++p) {
             const uint32_t hs = s.hs0 + 2u * (uint32_t)sw + (uint32_t)p;

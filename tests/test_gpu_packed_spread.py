@@ -1,7 +1,9 @@
-"""Packed sweeps on either side of the rule that spreads groups over the GPU
-(fewer than two full blocks per SM: 304 on the 152 SMs of GB300), with ragged
-last groups, and lattices whose last 32-site chunk of the gather is partial.
-Spins, energies and parents bit-exact against the oracle."""
+"""Packed sweeps on either side of the rules that choose their shape on a GPU of
+152 SMs: a team of threads per word (few threads to an SM; populations of a few
+thousand, as in most other tests, take it), groups spread over the SMs (fewer
+than two full blocks per SM), full blocks.  Ragged last groups, lattices whose
+last 32-site chunk of the gather is partial, and temperatures of every
+comparison mode.  Spins, energies and parents bit-exact against the oracle."""
 import numpy as np
 import pytest
 
@@ -12,11 +14,12 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("D,L,R,layout", [
     (3, 4, 64 * 2424 - 5, 1), (3, 4, 64 * 2425 + 1, 1), (3, 4, 64 * 607 + 9, 2), (3, 4, 64 * 609 - 1, 1),
+    (3, 4, 64 * 608, 1), (3, 6, 64 * 152 - 3, 1), (3, 6, 64 * 153, 1), (3, 8, 64 * 152, 2), (3, 8, 64 * 153 - 1, 1),
     (2, 2, 64 * 700 + 3, 1), (3, 6, 64 * 609 + 33, 1), (2, 6, 64 * 610 + 1, 1), (2, 10, 64 * 20 + 7, 1),
 ])
 def test_packed_spread(pa, oracle, D, L, R, layout):
     P = pa
-    J, betas = W.couplings_pm(D, L, 300 + L), np.array([0.0, 0.5, 0.9])
+    J, betas = W.couplings_pm(D, L, 300 + L), np.array([0.0, 0.5, 1.3, 3.2, 4.8])
     ref = oracle.Sim(D, L, 0, J, None, R, betas, 1, 71)
     pop = P.Population(D, L, 0, J, None, R, betas, 1, 71, layout=layout)
     try:
