@@ -7,8 +7,9 @@
 
 namespace pa {
 
-// Block b takes GPB groups; with `spread` the groups are spread evenly over the
-// grid instead (at most GPB a block).
+// Block b takes GPB groups; with spread > 0 the groups are spread evenly instead:
+// every SM gets an even share (blocks b, b + spread, ... run on one SM), and that
+// is split over its blocks (at most GPB a block).
 template <int D, int L, int GPB, int THREADS, bool I8, bool SHARD = false>
 __global__ void __launch_bounds__(THREADS, 4) sweep_packed_kernel(PackedSweepArgs a, int spread)
 {
@@ -16,8 +17,10 @@ __global__ void __launch_bounds__(THREADS, 4) sweep_packed_kernel(PackedSweepArg
     const int G = packed_groups(a.i);
     int g0 = blockIdx.x * GPB, gend = min(g0 + GPB, G);
     if (GPB > 1 && spread) {
-        g0 = (int)((long long)G * blockIdx.x / gridDim.x);
-        gend = (int)((long long)G * (blockIdx.x + 1) / gridDim.x);
+        const int sm = blockIdx.x % spread, slot = blockIdx.x / spread, slots = (gridDim.x - sm + spread - 1) / spread;
+        const int a0 = (int)((long long)G * sm / spread), a1 = (int)((long long)G * (sm + 1) / spread);
+        g0 = a0 + (a1 - a0) * slot / slots;
+        gend = a0 + (a1 - a0) * (slot + 1) / slots;
     }
     sweep_packed_tile<D, L, GPB, THREADS, I8, true, SHARD>(a.s, a.i, g0, gend, smem_packed);
 }
@@ -97,18 +100,24 @@ static cudaError_t launch_dl(const PackedSweepArgs& a, int gpb, int threads, cud
         if ((long long)a.i.G * team_threads<D, L>() <= (long long)sms * per_sm)
             return i8 ? launch_team<D, L, true>(a, st) : launch_team<D, L, false>(a, st);
     }
-    // fewer than two full blocks to an SM: spread the groups over up to four
-    // blocks to an SM (L=6, R=40001: 119 -> 81 us; L=6, R=5000: 116 -> 41 us;
-    // 2D L=16, R=30000: 125 -> 68 us); with more full blocks than that spreading
-    // measured 2 to 5 % slower (L=8, R=10^5: 213 -> 218 us)
+    // less than a wave of full blocks (four to an SM): an SM with one block more
+    // than another sets the time, so the groups are spread evenly over as many
+    // blocks to an SM as full ones would need, at least two (us a launch, full
+    // blocks -> spread: L=6, R=40001 111 -> 74; L=6, R=2x10^5 213 -> 188; L=8,
+    // R=5x10^4 149 -> 126; L=8, R=1.2x10^5 260 -> 232; 2D L=16, R=6x10^4 116 -> 88).
+    // Tiles with late compaction lose more to their partly filled queue rounds
+    // than the balance gives when the blocks would be four fifths full (L=8,
+    // R=10^5: 205 -> 209; R=1.5x10^5: 268 -> 272)
     int spread = 0;
     if constexpr (s.gpb > 1) {
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (grid < 2 * sms) {
-            spread = 1;
-            grid = a.i.G < 4 * sms ? a.i.G : 4 * sms;
+        const int k = grid <= 2 * sms ? 2 : (grid + sms - 1) / sms;
+        const long long room = (long long)k * sms * s.gpb;
+        if (grid < 4 * sms && (!PackedShape<D, L, s.gpb, s.threads>::kLate || 10ll * a.i.G < 8 * room)) {
+            grid = a.i.G < k * sms ? a.i.G : k * sms;
+            spread = grid < sms ? grid : sms;
         }
     }
     return i8 ? launch_one<D, L, s.gpb, s.threads, true>(a, grid, spread, st)

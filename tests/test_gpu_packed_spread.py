@@ -1,7 +1,8 @@
 """Packed sweeps on either side of the rules that choose their shape on a GPU of
 152 SMs: a team of threads per word (few threads to an SM; populations of a few
-thousand, as in most other tests, take it), groups spread over the SMs (fewer
-than two full blocks per SM), full blocks.  Ragged last groups, lattices whose
+thousand, as in most other tests, take it), groups spread evenly over the SMs
+(less than a wave of full blocks; with late compaction only if they would be
+less than four fifths full), full blocks.  Ragged last groups, lattices whose
 last 32-site chunk of the gather is partial, and temperatures of every
 comparison mode.  Spins, energies and parents bit-exact against the oracle."""
 import numpy as np
@@ -15,6 +16,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("D,L,R,layout", [
     (3, 4, 64 * 2424 - 5, 1), (3, 4, 64 * 2425 + 1, 1), (3, 4, 64 * 607 + 9, 2), (3, 4, 64 * 609 - 1, 1),
     (3, 4, 64 * 608, 1), (3, 6, 64 * 152 - 3, 1), (3, 6, 64 * 153, 1), (3, 8, 64 * 152, 2), (3, 8, 64 * 153 - 1, 1),
+    (3, 4, 64 * 4864 - 7, 1), (3, 4, 64 * 4865, 1), (3, 8, 64 * 972, 1), (3, 8, 64 * 973 - 2, 1),
     (2, 2, 64 * 700 + 3, 1), (3, 6, 64 * 609 + 33, 1), (2, 6, 64 * 610 + 1, 1), (2, 10, 64 * 20 + 7, 1),
 ])
 def test_packed_spread(pa, oracle, D, L, R, layout):
