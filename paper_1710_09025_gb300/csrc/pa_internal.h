@@ -247,18 +247,16 @@ cudaError_t launch_resample_batched(const ResampleArgs* tab, int n_inst, int max
 
 struct ObsPartial {
     long long sumE, sumE2, min_lo, min_hi;
-    double sumEd, sumE2d, clnc, pad;
+    double sumEd, sumE2d;
+    long long chi, clo;          // sum of c ln c over families: chi 2^-20 + clo 2^-52
 };
 constexpr int kObsBlocks = 608;  // most blocks of the observables reduction (4 per SM of GB300)
 // blocks of the observables reduction for a population of R (a function of R
 // only, non-decreasing, so that a grid sized for a capacity covers any smaller
-// population): about 4096 replicas each, but at least min(ceil(R / 1024), 304)
-// blocks, so that small populations spread their FP64 work over many SMs
-// (R = 10^5: 0.048 -> 0.026 ms per step), at most kObsBlocks
+// population): one per 256 replicas, at most kObsBlocks
 __host__ __device__ constexpr inline int obs_blocks(int R)
 {
-    const int a = (R + 4095) / 4096, b = (R + 1023) / 1024 < 304 ? (R + 1023) / 1024 : 304;
-    const int n = a > b ? a : b;
+    const int n = (R + 255) / 256;
     return n < 1 ? 1 : (n > kObsBlocks ? kObsBlocks : n);
 }
 struct ObsArgs {
@@ -268,12 +266,12 @@ struct ObsArgs {
     const longlong2* E128;
     const int32_t* family;
     ObsPartial* part;            // [kObsBlocks] scratch
-    const double* logc;          // [kLogC] log(c) for the family entropy (or null)
+    const double* logc;          // [kLogC] c ln c for the family entropy
     StepAcc* cur;
     int* sync;                   // zeroed block counter: the last block combines
 };
-// family sizes below kLogC take log(c) from a table that the context fills
-// once with the same device log; larger ones evaluate it
+// family sizes below kLogC take c ln c from a table that the context fills
+// once with the same device arithmetic; larger ones evaluate it
 constexpr int kLogC = 4096;
 cudaError_t launch_logc_table(double* t, cudaStream_t st);
 cudaError_t launch_observe(const ObsArgs& a, cudaStream_t st);

@@ -35,19 +35,19 @@ __device__ __forceinline__ double e_minus_min_to_double(const ResampleArgs& a, i
 
 // true in the block that finishes last (each of n_blocks calls it once); the
 // counter is reset for the next launch.  Writes before the call are visible
-// to the last block (fence before the count).
+// to the last block: one acquire-release addition after the block's barrier
+// (a fence on each side of a relaxed one took about 1 us more).
 __device__ __forceinline__ bool last_block(int* counter, int n_blocks)
 {
     __shared__ int s_last;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        const int done = atomicAdd(counter, 1);
+        int done;
+        asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(done) : "l"(counter) : "memory");
         s_last = done == n_blocks - 1;
         if (s_last) *counter = 0;
     }
     __syncthreads();
-    if (s_last) __threadfence();
     return s_last;
 }
 
@@ -135,33 +135,33 @@ __device__ __forceinline__ void rs_levels_body(const ResampleArgs& a, int b, int
     __syncthreads();
     const int nruns = (n + kFan - 1) / kFan;
     if (warp == 0) {
+        // run `lane`, left to right (starting from +0 and adding +0 past the end
+        // changes nothing: the sums are not negative)
+        double* x = s_w + lane * (kFan + 1);
+        const int cnt = min(kFan, n - lane * kFan);
         double tot = 0.0;
-        if (lane < nruns) {  // run `lane`, left to right
-            double* x = s_w + lane * (kFan + 1);
-            const int cnt = min(kFan, n - lane * kFan);
-            double acc = 0.0;
-            for (int j0 = 0; j0 < cnt; j0 += 8) {
-                double v[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = j0 + j < cnt ? x[j0 + j] : 0.0;
+        for (int j0 = 0; j0 < kFan; j0 += 8) {
+            double v[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (j0 + j < cnt) {
-                        acc = (j0 + j == 0) ? v[0] : __dadd_rn(acc, v[j]);
-                        x[j0 + j] = acc;
-                    }
-                }
-            }
-            tot = acc;
-            s_t[lane] = acc;
+            for (int j = 0; j < 8; ++j) v[j] = j0 + j < cnt ? x[j0 + j] : 0.0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = tot = __dadd_rn(tot, v[j]);
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (j0 + j < cnt) x[j0 + j] = v[j];
         }
+        s_t[lane] = tot;  // 0 past the last run
         __syncwarp();
         if (lane == 0) {  // the block's run totals, left to right
-            double acc = n > 0 ? s_t[0] : 0.0;
-            s_l1[0] = acc;
-            for (int c = 1; c < nruns; ++c) {
-                acc = __dadd_rn(acc, s_t[c]);
-                s_l1[c] = acc;
+            double acc = 0.0;
+#pragma unroll
+            for (int c0 = 0; c0 < kFan; c0 += 8) {
+                double v[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) v[c] = s_t[c0 + c];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) s_l1[c0 + c] = acc = __dadd_rn(acc, v[c]);
             }
             a.upper[b] = acc;
         }
@@ -296,10 +296,7 @@ __device__ __forceinline__ void rs_top_levels(double* up, int nb)
 #pragma unroll
                 for (int j = 0; j < 8; ++j) v[j] = j0 + j < cnt ? x[j0 + j] : 0.0;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    acc = (j0 + j == 0) ? v[0] : __dadd_rn(acc, v[j]);  // +0 past the run: no change
-                    v[j] = acc;
-                }
+                for (int j = 0; j < 8; ++j) v[j] = acc = __dadd_rn(acc, v[j]);  // +0 first and past the run: no change
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
                     if (j0 + j < cnt) x[j0 + j] = v[j];
@@ -500,6 +497,31 @@ __device__ __forceinline__ int first_of_32(Pred pred)
     lo += q1 ? 0 : q3 ? 2 : q5 ? 4 : 6;
     return pred(lo) ? lo : lo + 1;
 }
+// v 2^-53 for v < 2^53, exactly, as the double's bits: integer work instead of
+// an FP64 conversion and product
+__device__ __forceinline__ double uniform53_int(uint32_t hi, uint32_t lo)
+{
+    const unsigned long long v = (unsigned long long)(hi >> 5) << 26 | (lo >> 6);
+    if (v == 0) return 0.0;
+    const int lz = __clzll((long long)v);
+    return __longlong_as_double((long long)(((unsigned long long)(1032 - lz) << 52) + (v << (lz - 11))));
+}
+// The first i of run c (sums l_0 .. l_{n-1}, q before the run) with q + l_i past x.
+// q + l_i does not decrease with i and x - q, rounded, is within a unit of the
+// sum that reaches x, so the search compares l_i with it (integer compares of the
+// bit patterns) and the specified sums settle the last step or two: two or three
+// FP64 additions a draw instead of seven (GB300 has few FP64 units).
+template <class Past, class Load>
+__device__ __forceinline__ int rs_first_in_run(double q, long long x, int n, Past past, Load load)
+{
+    const long long t = dbits(__dsub_rn(__longlong_as_double(x), q));  // negative: below every sum
+    int i = first_of_32([&](int j) { return j >= n || dbits(load(j)) >= t; });
+    auto reached = [&](int j) { return past(dbits(__dadd_rn(q, load(j)))); };
+    i = min(i, n - 1);
+    while (i > 0 && reached(i - 1)) --i;
+    while (i < n - 1 && !reached(i)) ++i;
+    return i;
+}
 __device__ __forceinline__ void rs_draws_body(const ResampleArgs& a, int q0, int per)
 {
     __shared__ long long s_end[kMaxSeg];
@@ -520,7 +542,7 @@ __device__ __forceinline__ void rs_draws_body(const ResampleArgs& a, int q0, int
         const int q = q0 + d * nt + tid;
         if (q >= a.Rn) break;
         const u32x4 o = philox((uint32_t)q, (uint32_t)a.k, 0u, a.c3, a.key0, a.key1);
-        const long long x = dbits(__dmul_rn(uniform53(o.x, o.y), S));  // x >= 0
+        const long long x = dbits(__dmul_rn(uniform53_int(o.x, o.y), S));  // x >= 0
         int lo = 0, hi = nseg;  // first segment whose end exceeds x
         while (lo < hi) {
             const int mid = lo + ((hi - lo) >> 1);
@@ -540,13 +562,10 @@ __device__ __forceinline__ void rs_draws_body(const ResampleArgs& a, int q0, int
             const long long p = dbits(a.runP[b0 * kFan + t]);
             return strict ? x < p : p >= x;
         });
-        const double qc = a.runq[min(c, leaves - 1)];
-        const int i = c * kFan + first_of_32([&](int t) {
-            if (c * kFan + t >= R) return true;
-            const long long p = dbits(__dadd_rn(qc, a.P[c * kFan + t]));
-            return strict ? x < p : p >= x;
-        });
-        const int w = min(i, R - 1);
+        const int cc = min(c, leaves - 1), i0 = cc * kFan;
+        const int w = i0 + rs_first_in_run(a.runq[cc], x, min(kFan, R - i0),
+                                           [&](long long p) { return strict ? x < p : p >= x; },
+                                           [&](int t) { return a.P[i0 + t]; });
         atomicAdd(&a.counts[w], 1);
         if (hist) atomicAdd(&s_hist[w / sbits], 1);
         else atomicAdd(&a.bcount[w / sbits], 1);
@@ -618,7 +637,7 @@ __global__ void __launch_bounds__(kDrawThreads) rs_draws_batched(const ResampleA
 __device__ __forceinline__ int rs_nearest_copies(const ResampleArgs& a, int i, double S)
 {
     const u32x4 o = philox((uint32_t)i, (uint32_t)a.k, 1u, a.c3, a.key0, a.key1);
-    const double u = uniform53(o.x, o.y);
+    const double u = uniform53_int(o.x, o.y);
     const double tau = __ddiv_rn(__dmul_rn(a.target, a.w[i]), S);
     const double fl = floor(tau);
     return (int32_t)fl + (u < __dsub_rn(tau, fl) ? 1 : 0);
@@ -887,7 +906,7 @@ __global__ void __launch_bounds__(kWBlock) rs_cluster_kernel(ResampleArgs a)
     } else {
         for (int q = b * kWBlock + tid; q < a.Rn; q += gridDim.x * kWBlock) {
             const u32x4 o = philox((uint32_t)q, (uint32_t)a.k, 0u, a.c3, a.key0, a.key1);
-            const long long x = dbits(__dmul_rn(uniform53(o.x, o.y), S));  // x >= 0
+            const long long x = dbits(__dmul_rn(uniform53_int(o.x, o.y), S));  // x >= 0
             const bool strict = x < s_end[nb - 1];  // else x == S after rounding: the first P >= x
             auto past = [&](long long p) { return strict ? x < p : p >= x; };
             int bl = 0;
@@ -895,10 +914,8 @@ __global__ void __launch_bounds__(kWBlock) rs_cluster_kernel(ResampleArgs a)
             const int c = min(leaves - 1, bl * kFan + first_of_32([&](int t) {
                 return bl * kFan + t >= leaves || past(dbits(s_rp[bl * kFan + t]));
             }));
-            const double qc = s_rq[c];
-            const int i = min(R - 1, c * kFan + first_of_32([&](int t) {
-                return c * kFan + t >= R || past(dbits(__dadd_rn(qc, __ldcg(a.P + c * kFan + t))));
-            }));
+            const int i = c * kFan + rs_first_in_run(s_rq[c], x, min(kFan, R - c * kFan), past,
+                                                     [&](int t) { return __ldcg(a.P + c * kFan + t); });
             atomicAdd(&a.counts[i], 1);
             atomicAdd(&s_hist[i / kWBlock], 1);
         }
@@ -996,11 +1013,11 @@ cudaError_t launch_resample_batched(const ResampleArgs* tab, int n_inst, int max
     return cudaGetLastError();
 }
 
-// log(c) for c < kLogC (entries 0 and 1 are never read: a run of one adds 0)
+// c ln c for c < kLogC (entries 0 and 1 are never read: a run of one adds 0)
 __global__ void logc_table_kernel(double* t)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < kLogC) t[c] = c > 0 ? log((double)c) : 0.0;
+    if (c < kLogC) t[c] = c > 0 ? __dmul_rn((double)c, log((double)c)) : 0.0;
 }
 cudaError_t launch_logc_table(double* t, cudaStream_t st)
 {
@@ -1009,31 +1026,38 @@ cudaError_t launch_logc_table(double* t, cudaStream_t st)
 }
 
 // ---------------- observables (Sec. V.A, Eq. 9; Sec. II.B, Eq. 2) ----------------
-// kObsBlocks blocks each reduce a contiguous slice of the population in a
-// fixed order; one block combines the partials in block order.  The result
-// does not depend on the GPU (the partition depends only on R).
-// The launch is latency: one round of loads, then short chains.  A run of equal
-// family ids ends at the next start, found from the warp's ballot, the other
-// warps' first starts, and only for the last run of a 1024-replica window by a
-// search beyond it (the whole warp, 32 probes a round).
+// At most kObsBlocks blocks each reduce a contiguous slice of the population; the
+// last block to finish combines the partials.  Sums of +-J energies and the
+// family entropy's sum of c ln c are integers (a term is a double of at least 1,
+// so a multiple of 2^-52: two 64-bit sums hold every one exactly), the same in
+// any order and off the FP64 units; real-coupling energies are FP64 in a fixed
+// order.  The partition depends only on R, so the result does not depend on the
+// GPU.  The launch is latency: one round of loads, then short chains.  A run of
+// equal family ids ends at the next start, found from the warp's ballot, the
+// other warps' first starts, and only for the last run of a window by a search
+// beyond it (the whole warp, 32 probes a round).  R = 10^5: 15 -> XX us, 5 x 10^4
+// with real couplings 17 -> XX us (small blocks: the FP64 sums spread over the
+// SMs).
+constexpr int kObsThreads = 256;
+constexpr int kObsWarps = kObsThreads / 32;
 __device__ __forceinline__ void observe_partial_body(const ObsArgs& a)
 {
-    __shared__ long long s_ll[2][32];
-    __shared__ double s_d[3][32];
-    __shared__ __int128 s_min[32];
-    __shared__ int s_first[32];
+    __shared__ long long s_ll[4][kObsWarps];
+    __shared__ double s_d[2][kObsWarps];
+    __shared__ __int128 s_min[kObsWarps];
+    __shared__ int s_first[kObsWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R = a.Rdev ? *a.Rdev : a.R;
     const int nb = obs_blocks(R);
     if ((int)blockIdx.x >= nb) return;  // block-uniform
     const int per = (R + nb - 1) / nb;
     const int j0 = blockIdx.x * per, j1 = min(R, j0 + per);
-    long long se = 0, se2 = 0;
-    double sed = 0.0, se2d = 0.0, clnc = 0.0;
+    long long se = 0, se2 = 0, chi = 0, clo = 0;
+    double sed = 0.0, se2d = 0.0;
     int mn32 = 0x7fffffff;
     __int128 mn = (__int128)(((unsigned __int128)1 << 127) - 1);
-    for (int jb = j0; jb < j1; jb += 1024) {
-        const int j = jb + tid, jend = min(j1, jb + 1024);
+    for (int jb = j0; jb < j1; jb += kObsThreads) {
+        const int j = jb + tid, jend = min(j1, jb + kObsThreads);
         int f = 0, fprev = 0;
         if (j < j1) {
             f = a.family[j];
@@ -1058,7 +1082,7 @@ __device__ __forceinline__ void observe_partial_body(const ObsArgs& a)
         __syncthreads();
         if (bal) {  // warp-uniform
             // first start in a later warp, or beyond the window for the last run
-            int nxt = __reduce_min_sync(0xffffffffu, lane > warp ? s_first[lane] : 0x7fffffff);
+            int nxt = __reduce_min_sync(0xffffffffu, lane > warp && lane < kObsWarps ? s_first[lane] : 0x7fffffff);
             if (nxt == 0x7fffffff) {
                 const int fl = __shfl_sync(0xffffffffu, f, 31 - __clz(bal));
                 int lo = jend, hi = R;  // the first index in [lo, hi) of another family, else hi
@@ -1076,25 +1100,30 @@ __device__ __forceinline__ void observe_partial_body(const ObsArgs& a)
             if (start) {
                 const unsigned later = bal & ~((2u << lane) - 1u);
                 const int e = later ? jb + warp * 32 + __ffs(later) - 1 : nxt;
-                // c ln c of the run; a run of one adds exactly 0 (GB300's FP64 log
-                // is costly: short runs read it from the context's table, which
-                // holds the same device log of the same argument)
+                // c ln c of the run (a run of one adds 0; short runs read it from
+                // the context's table)
                 const int cn = e - j;
                 if (cn > 1) {
-                    const double c = (double)cn;
-                    const double lc = (a.logc && cn < kLogC) ? a.logc[cn] : log(c);
-                    clnc = __fma_rn(c, lc, clnc);
+                    const double c = (double)cn, v = cn < kLogC ? a.logc[cn] : __dmul_rn(c, log(c));
+                    // v = m 2^(x - 52), 0 <= x < 31: high part in units of 2^-20, low 32 bits below
+                    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+                    const int x = (int)(bits >> 52) - 1023;
+                    const unsigned long long m = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+                    chi += (long long)(m >> (32 - x));
+                    clo += (long long)((m << x) & 0xFFFFFFFFull);
                 }
             }
         }
         __syncthreads();  // s_first is rewritten by the next window
     }
-    // fixed shuffle trees; the FP64 ones only where they can add something
-    // (GB300 has little FP64 throughput): +-J energies are integer sums, and a
-    // warp without a family start has clnc = 0 in every lane
+    // fixed shuffle trees
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        chi += __shfl_down_sync(0xffffffffu, chi, off);
+        clo += __shfl_down_sync(0xffffffffu, clo, off);
+    }
     if (a.kind == 0) {
-        mn32 = __reduce_min_sync(0xffffffffu, mn32);
-        mn = mn32;
+        mn = __reduce_min_sync(0xffffffffu, mn32);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             se += __shfl_down_sync(0xffffffffu, se, off);
@@ -1111,104 +1140,101 @@ __device__ __forceinline__ void observe_partial_body(const ObsArgs& a)
             if (o < mn) mn = o;
         }
     }
-    if (__any_sync(0xffffffffu, clnc != 0.0)) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) clnc = __dadd_rn(clnc, __shfl_down_sync(0xffffffffu, clnc, off));
-    }
     if (lane == 0) {
-        s_ll[0][warp] = se; s_ll[1][warp] = se2;
-        s_d[0][warp] = sed; s_d[1][warp] = se2d; s_d[2][warp] = clnc;
+        s_ll[0][warp] = se; s_ll[1][warp] = se2; s_ll[2][warp] = chi; s_ll[3][warp] = clo;
+        s_d[0][warp] = sed; s_d[1][warp] = se2d;
         s_min[warp] = mn;
     }
     __syncthreads();
-    if (warp != 0) return;
     ObsPartial& p = a.part[blockIdx.x];
-    if (a.kind == 0) {
-        se = s_ll[0][lane]; se2 = s_ll[1][lane];
+    if (tid < 4) {
+        long long v = 0;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            se += __shfl_down_sync(0xffffffffu, se, off);
-            se2 += __shfl_down_sync(0xffffffffu, se2, off);
-        }
-        const int m = __reduce_min_sync(0xffffffffu, (int)s_min[lane]);
-        if (lane == 0) { p.sumE = se; p.sumE2 = se2; p.min_lo = m; p.min_hi = m < 0 ? -1 : 0; }
-    } else if (lane == 3) {
+        for (int w = 0; w < kObsWarps; ++w) v += s_ll[tid][w];
+        if (tid == 0) p.sumE = v;
+        else if (tid == 1) p.sumE2 = v;
+        else if (tid == 2) p.chi = v;
+        else p.clo = v;
+    } else if (tid >= 32 && tid < 34) {  // the warps' FP64 sums in warp order
+        double v = s_d[tid - 32][0];
+        if (a.kind != 0)
+#pragma unroll
+            for (int w = 1; w < kObsWarps; ++w) v = __dadd_rn(v, s_d[tid - 32][w]);
+        if (tid == 32) p.sumEd = v;
+        else p.sumE2d = v;
+    } else if (tid == 64) {
         __int128 M = s_min[0];
-        for (int w = 1; w < 32; ++w)
+#pragma unroll
+        for (int w = 1; w < kObsWarps; ++w)
             if (s_min[w] < M) M = s_min[w];
-        p.sumE = 0; p.sumE2 = 0;
         p.min_lo = (long long)(unsigned long long)M;
         p.min_hi = (long long)(M >> 64);
     }
-    if (lane < 3) {  // the warps' FP64 sums in warp order, one chain per lane (+0 first: no change)
-        double acc = 0.0;
-        if (lane == 2 || a.kind != 0)
-            for (int w = 0; w < 32; ++w) acc = __dadd_rn(acc, s_d[lane][w]);
-        if (lane == 0) p.sumEd = acc;
-        else if (lane == 1) p.sumE2d = acc;
-        else p.clnc = acc;
-    }
 }
-__device__ __forceinline__ void observe_final_body(const ObsArgs& a);
-__global__ void __launch_bounds__(1024) observe_partial_kernel(ObsArgs a)
-{
-    observe_partial_body(a);
-    const int nb = obs_blocks(a.Rdev ? *a.Rdev : a.R);
-    if ((int)blockIdx.x < nb && last_block(a.sync, nb) && threadIdx.x < 32) observe_final_body(a);  // combine in a fixed order
-}
-__global__ void __launch_bounds__(1024) observe_partial_batched(const ObsArgs* tab)
-{
-    const ObsArgs& a = tab[blockIdx.y];
-    observe_partial_body(a);
-    const int nb = obs_blocks(a.R);
-    if ((int)blockIdx.x < nb && last_block(a.sync, nb) && threadIdx.x < 32) observe_final_body(a);
-}
-
 // partials combined by one warp: lane l adds blocks l, l + 32, ... in order,
 // then the 32 lane sums are added by a fixed shuffle tree (the same order on
 // every GPU)
 __device__ __forceinline__ void observe_final_body(const ObsArgs& a)
 {
     const int lane = threadIdx.x & 31;
-    long long A = 0, B = 0;
-    double C = 0.0, Dd = 0.0, F = 0.0;
+    long long A = 0, B = 0, H = 0, Lw = 0;
+    double C = 0.0, Dd = 0.0;
     __int128 M = (__int128)(((unsigned __int128)1 << 127) - 1);
     const int nb = obs_blocks(a.Rdev ? *a.Rdev : a.R);
     for (int b = lane; b < nb; b += 32) {
-        const ObsPartial p = a.part[b];
-        A += p.sumE; B += p.sumE2;
-        C = __dadd_rn(C, p.sumEd); Dd = __dadd_rn(Dd, p.sumE2d); F = __dadd_rn(F, p.clnc);
-        const __int128 m = ((__int128)p.min_hi << 64) | (unsigned long long)p.min_lo;
+        const ObsPartial* p = a.part + b;
+        A += __ldcg(&p->sumE); B += __ldcg(&p->sumE2);
+        H += __ldcg(&p->chi); Lw += __ldcg(&p->clo);
+        if (a.kind != 0) {
+            C = __dadd_rn(C, __ldcg(&p->sumEd));
+            Dd = __dadd_rn(Dd, __ldcg(&p->sumE2d));
+        }
+        const __int128 m = ((__int128)__ldcg(&p->min_hi) << 64) | (unsigned long long)__ldcg(&p->min_lo);
         if (m < M) M = m;
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         A += __shfl_down_sync(0xffffffffu, A, off);
         B += __shfl_down_sync(0xffffffffu, B, off);
-        C = __dadd_rn(C, __shfl_down_sync(0xffffffffu, C, off));
-        Dd = __dadd_rn(Dd, __shfl_down_sync(0xffffffffu, Dd, off));
-        F = __dadd_rn(F, __shfl_down_sync(0xffffffffu, F, off));
+        H += __shfl_down_sync(0xffffffffu, H, off);
+        Lw += __shfl_down_sync(0xffffffffu, Lw, off);
         const long long lo = __shfl_down_sync(0xffffffffu, (long long)(unsigned long long)M, off);
         const long long hi = __shfl_down_sync(0xffffffffu, (long long)(M >> 64), off);
         const __int128 o = ((__int128)hi << 64) | (unsigned long long)lo;
         if (o < M) M = o;
     }
+    if (a.kind != 0) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            C = __dadd_rn(C, __shfl_down_sync(0xffffffffu, C, off));
+            Dd = __dadd_rn(Dd, __shfl_down_sync(0xffffffffu, Dd, off));
+        }
+    }
     if (lane != 0) return;
     a.cur->sumE = A; a.cur->sumE2 = B;
     a.cur->sumEd = C; a.cur->sumE2d = Dd;
-    a.cur->sum_clnc = F;
+    a.cur->sum_clnc = __dmul_rn(i128_to_double(((__int128)H << 32) + Lw), 0x1p-52);
     a.cur->emin_lo = (long long)(unsigned long long)M;
     a.cur->emin_hi = (long long)(M >> 64);
 }
+__device__ __forceinline__ void observe_launch(const ObsArgs& a)
+{
+    observe_partial_body(a);
+    const int nb = obs_blocks(a.Rdev ? *a.Rdev : a.R);
+    if ((int)blockIdx.x < nb && last_block(a.sync, nb) && threadIdx.x < 32) observe_final_body(a);
+}
+__global__ void __launch_bounds__(kObsThreads) observe_kernel(ObsArgs a) { observe_launch(a); }
+__global__ void __launch_bounds__(kObsThreads) observe_batched(const ObsArgs* tab) { observe_launch(tab[blockIdx.y]); }
+
 cudaError_t launch_observe(const ObsArgs& a, cudaStream_t st)
 {
-    observe_partial_kernel<<<obs_blocks(a.R), 1024, 0, st>>>(a);
+    observe_kernel<<<obs_blocks(a.R), kObsThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_observe_batched(const ObsArgs* tab, int n_inst, int maxR, cudaStream_t st)
 {
-    observe_partial_batched<<<dim3(obs_blocks(maxR), (unsigned)n_inst), 1024, 0, st>>>(tab);
+    observe_batched<<<dim3(obs_blocks(maxR), (unsigned)n_inst), kObsThreads, 0, st>>>(tab);
     return cudaGetLastError();
 }
 
