@@ -19,6 +19,8 @@
 #include "pa_device.cuh"
 #include "pa_internal.h"
 
+#include <atomic>
+
 namespace pa {
 
 __device__ __forceinline__ __int128 ll2_to_i128(longlong2 v)
@@ -65,25 +67,25 @@ __device__ __forceinline__ int rs_src(const ResampleArgs& a) { return a.Rsrc ? *
 // evaluates each level's weight once (spec_exp64 of the same argument) and looks
 // the weights up.
 //
-// Two shapes.  Populations of at most kFuseR: 1024 threads, one weight each, and
-// the last block to finish completes the prefix, the run search table and S
-// (rs_fused): with at most 128 blocks the launch is latency alone, and a second
-// and third launch cost more than one SM's work.  Larger ones: 256 threads, so
+// Two shapes (and the cluster below).  Populations of at most kFuseR: the last
+// block to finish sums levels 1 and up and completes the run search table and S
+// (rs_fused): a second and third launch cost more than one SM's work.  Blocks of
+// 1024 weights with +-J, where a block evaluates few exponentials and more warps
+// serve the last block; of 256 with real couplings, so that the exponentials (one
+// per replica) spread over the SMs.  Larger ones: 1024 weights and 256 threads, so
 // that several blocks' dependent FP64 chains overlap on an SM, and the run table
-// is its own launch (rs_runs_kernel).  R = 10^5, by ncu: level table + weights +
-// finalize 24 us -> 16 us, most of it 62-cycle FP64 additions in a chain.
+// is its own launch (rs_runs_kernel).  By ncu: +-J R = 10^5 level table + weights +
+// finalize 24 us -> 14.3 (blocks of 256: 16.9), most of it 62-cycle FP64 additions
+// in a chain; real couplings R = 5 x 10^4 20.2 us in blocks of 1024, 16.8 of 256.
 constexpr int kFuseR = 128 * kWBlock;
-template <int T>
-__device__ __forceinline__ void rs_levels_body(const ResampleArgs& a, int b, int R, int emin)
+// weights of replicas i0 + tid + j T, j < PER (those below i0 + n), into w; tab:
+// PER T doubles of shared memory; also to a.w for the nearest-integer scheme
+template <int T, int PER>
+__device__ __forceinline__ void rs_block_weights(const ResampleArgs& a, int i0, int n, int emin, double (&w)[PER],
+                                                 double* tab)
 {
-    constexpr int PER = kWBlock / T;
-    __shared__ double s_w[kFan * (kFan + 1)];  // run c at [c (kFan + 1)], padded against bank conflicts
-    __shared__ double s_t[kFan], s_l1[kFan];
     __shared__ int s_lo[T / 32], s_hi[T / 32];
-    const int i0 = b * kWBlock;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n = min(kWBlock, R - i0);
-    if (tid == 0 && a.bcount && b < rs_scan_blocks(R)) a.bcount[b] = 0;
     if (a.kind == 0) {
         int lv[PER], lo = 0x7fffffff, hi = -1;
 #pragma unroll
@@ -101,73 +103,101 @@ __device__ __forceinline__ void rs_levels_body(const ResampleArgs& a, int b, int
         __syncthreads();
         lo = __reduce_min_sync(0xffffffffu, lane < T / 32 ? s_lo[lane] : 0x7fffffff);
         hi = __reduce_max_sync(0xffffffffu, lane < T / 32 ? s_hi[lane] : -1);
-        // levels lo/4 .. hi/4 evaluated once each (staged in s_w, read before the weights replace them)
-        const int nlev = hi < 0x7ffffff0 && lo >= 0 ? (hi >> 2) - (lo >> 2) + 1 : kWBlock;
-        double w[PER];
-        if (nlev <= kWBlock / 2) {
+        // levels lo/4 .. hi/4 evaluated once each
+        const int nlev = hi < 0x7ffffff0 && lo >= 0 ? (hi >> 2) - (lo >> 2) + 1 : PER * T;
+        if (nlev <= PER * T / 2) {
             for (int t = tid; t < nlev; t += T)
-                s_w[t] = spec_exp64(-__dmul_rn(a.dbeta, (double)(4 * ((lo >> 2) + t))));
+                tab[t] = spec_exp64(-__dmul_rn(a.dbeta, (double)(4 * ((lo >> 2) + t))));
             __syncthreads();
 #pragma unroll
-            for (int j = 0; j < PER; ++j) w[j] = lv[j] >= 0 ? s_w[(lv[j] >> 2) - (lo >> 2)] : 0.0;
+            for (int j = 0; j < PER; ++j) w[j] = lv[j] >= 0 ? tab[(lv[j] >> 2) - (lo >> 2)] : 0.0;
         } else {
 #pragma unroll
             for (int j = 0; j < PER; ++j)
                 w[j] = tid + j * T < n ? spec_exp64(-__dmul_rn(a.dbeta, (double)lv[j])) : 0.0;
         }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            const int t = tid + j * T;
-            if (t < n) s_w[(t / kFan) * (kFan + 1) + t % kFan] = w[j];
-            if (t < n && a.scheme == 1) a.w[i0 + t] = w[j];
-        }
     } else {
 #pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            const int t = tid + j * T;
-            if (t >= n) continue;
-            const double w = spec_exp64(-__dmul_rn(a.dbeta, e_minus_min_to_double(a, i0 + t)));
-            if (a.scheme == 1) a.w[i0 + t] = w;
-            s_w[(t / kFan) * (kFan + 1) + t % kFan] = w;
-        }
+        for (int j = 0; j < PER; ++j)
+            w[j] = tid + j * T < n ? spec_exp64(-__dmul_rn(a.dbeta, e_minus_min_to_double(a, i0 + tid + j * T))) : 0.0;
+    }
+    if (a.scheme == 1) {
+#pragma unroll
+        for (int j = 0; j < PER; ++j)
+            if (tid + j * T < n) a.w[i0 + tid + j * T] = w[j];
+    }
+}
+// Sum of a run of cnt <= kFan weights at x, left to right, the sums left in place
+// (starting from +0 and adding +0 past the end changes nothing: no sum is
+// negative).  By whole warps.  The barriers keep the loads and stores out of the
+// chain of additions: stored one by one between them they hold up the next
+// addition (32 additions by one warp 3500 cycles, with the barriers 2260).
+__device__ __forceinline__ double rs_run_sums(double* x, int cnt)
+{
+    double tot = 0.0;
+#pragma unroll
+    for (int j0 = 0; j0 < kFan; j0 += 8) {
+        if (j0 > 0 && !__any_sync(0xffffffffu, j0 < cnt)) break;
+        double v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = j0 + j < cnt ? x[j0 + j] : 0.0;
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = tot = __dadd_rn(tot, v[j]);
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (j0 + j < cnt) x[j0 + j] = v[j];
+    }
+    return tot;
+}
+// the sums of the warp's values, left to right: lane l gets that of lanes 0 .. l
+template <int N>
+__device__ __forceinline__ double rs_lane_sums(double mine)
+{
+    const int lane = threadIdx.x & 31;
+    double acc = 0.0, res = 0.0;
+#pragma unroll
+    for (int c0 = 0; c0 < N; c0 += 8) {
+        double v[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) v[c] = __shfl_sync(0xffffffffu, mine, c0 + c);
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 8; ++c) v[c] = acc = __dadd_rn(acc, v[c]);
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (lane == c0 + c) res = v[c];
+    }
+    return res;
+}
+// a weights block of kWBlock weights by T threads: levels 0 and 1
+template <int T>
+__device__ __forceinline__ void rs_levels_body(const ResampleArgs& a, int b, int R, int emin)
+{
+    constexpr int PER = kWBlock / T;
+    __shared__ double s_w[kFan * (kFan + 1)];  // run c at [c (kFan + 1)], padded against bank conflicts
+    const int i0 = b * kWBlock;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = min(kWBlock, R - i0);
+    if (tid == 0 && a.bcount && b < rs_scan_blocks(R)) a.bcount[b] = 0;
+    double w[PER];
+    rs_block_weights<T, PER>(a, i0, n, emin, w, s_w);
+    __syncthreads();  // the level table in s_w has been read
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int t = tid + j * T;
+        if (t < n) s_w[(t / kFan) * (kFan + 1) + t % kFan] = w[j];
     }
     __syncthreads();
     const int nruns = (n + kFan - 1) / kFan;
     if (warp == 0) {
-        // run `lane`, left to right (starting from +0 and adding +0 past the end
-        // changes nothing: the sums are not negative)
-        double* x = s_w + lane * (kFan + 1);
-        const int cnt = min(kFan, n - lane * kFan);
-        double tot = 0.0;
-#pragma unroll
-        for (int j0 = 0; j0 < kFan; j0 += 8) {
-            double v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = j0 + j < cnt ? x[j0 + j] : 0.0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = tot = __dadd_rn(tot, v[j]);
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (j0 + j < cnt) x[j0 + j] = v[j];
-        }
-        s_t[lane] = tot;  // 0 past the last run
-        __syncwarp();
-        if (lane == 0) {  // the block's run totals, left to right
-            double acc = 0.0;
-#pragma unroll
-            for (int c0 = 0; c0 < kFan; c0 += 8) {
-                double v[8];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) v[c] = s_t[c0 + c];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) s_l1[c0 + c] = acc = __dadd_rn(acc, v[c]);
-            }
-            a.upper[b] = acc;
-        }
-        __syncwarp();
+        const double tot = rs_run_sums(s_w + lane * (kFan + 1), min(kFan, n - lane * kFan));
+        const double l1 = rs_lane_sums<kFan>(tot);  // the block's run totals (0 past the last)
+        if (lane == 31) a.upper[b] = l1;
         if (lane < nruns) {
-            a.lev1[b * kFan + lane] = s_l1[lane];
+            a.lev1[b * kFan + lane] = l1;
             if (a.runP) a.runP[b * kFan + lane] = tot;
         }
     }
@@ -210,26 +240,54 @@ __device__ __forceinline__ long long rs_run_table(const ResampleArgs& a, int b, 
 }
 
 __device__ __forceinline__ void rs_top_levels(double* up, int nb);
-// the last weights block of a population of at most kFuseR: levels >= 2 of the
-// prefix, run table, running maximum over the blocks, S
+// the last sub-block of a population of at most kFuseR: levels 1 and up of the
+// prefix, run table, running maximum over the weights blocks, S
+constexpr int kFuseBlocks = kFuseR / kWBlock;
+template <int T>
 __device__ __forceinline__ void rs_fused(const ResampleArgs& a, int R)
 {
-    constexpr int kNb = kFuseR / kWBlock;
+    // run totals, then the level-1 sums, of weights block b at [b (kFan + 1)]
+    __shared__ double s_l1[kFuseBlocks * (kFan + 1)];
     __shared__ double s_up[rs_upper_size(kFuseR)];
-    __shared__ long long s_bm[kNb];
+    __shared__ long long s_bm[kFuseBlocks];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nb = rs_wblocks(R);
-    for (int t = tid; t < nb; t += blockDim.x) s_up[t] = __ldcg(a.upper + t);
-    if (tid < kNb) s_bm[tid] = 0;
+    const int nb = rs_wblocks(R), leaves = rs_leaves(R);
+    for (int t = tid; t < nb * kFan; t += T)
+        s_l1[(t / kFan) * (kFan + 1) + t % kFan] = t < leaves ? __ldcg(a.runP + t) : 0.0;
+    if (tid < kFuseBlocks) s_bm[tid] = 0;
+    __syncthreads();
+    if (warp < (nb + 31) / 32) {
+        const double tot = rs_run_sums(s_l1 + tid * (kFan + 1), tid < nb ? kFan : 0);
+        if (tid < nb) s_up[tid] = tot;
+    }
     __syncthreads();
     rs_top_levels(s_up, nb);
-    for (int b = warp; b < nb; b += blockDim.x / 32) {
-        const long long m = rs_run_table(a, b, R, s_up);
-        if (lane == 0) s_bm[b] = m;
+    double next = warp * kFan + lane < leaves ? __ldcg(a.runP + warp * kFan + lane) : 0.0;
+    for (int b = warp; b < nb; b += T / 32) {
+        const int c = b * kFan + lane;
+        const double tot = next;
+        next = c + T < leaves ? __ldcg(a.runP + c + T) : 0.0;
+        const int pb = lane > 0 ? b : b - 1;  // block of run c - 1
+        double q = 0.0;
+        if (c > 0) {
+            const double l1 = s_l1[pb * (kFan + 1) + (lane > 0 ? lane - 1 : kFan - 1)];
+            q = pb == 0 ? l1 : __dadd_rn(s_up[pb - 1], l1);
+        }
+        long long m = c < leaves ? dbits(c == 0 ? tot : __dadd_rn(q, tot)) : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long u = __shfl_up_sync(0xffffffffu, m, o);
+            if (lane >= o) m = max(m, u);
+        }
+        if (c < leaves) {
+            a.runq[c] = q;
+            a.runP[c] = __longlong_as_double(m);
+        }
+        if (lane == 31) s_bm[b] = m;
     }
     __syncthreads();
     if (warp == 0) {
-        constexpr int PER = kNb / 32;
+        constexpr int PER = kFuseBlocks / 32;
         long long v[PER], m = 0;
 #pragma unroll
         for (int j = 0; j < PER; ++j) { m = max(m, s_bm[lane * PER + j]); v[j] = m; }
@@ -249,6 +307,31 @@ __device__ __forceinline__ void rs_fused(const ResampleArgs& a, int R)
         if (lane == 31) a.cur->S = __longlong_as_double(inc);
     }
 }
+// a sub-block: its weights and the sums inside its eight runs
+template <int T>
+__global__ void __launch_bounds__(T) rs_weights_fused_kernel(ResampleArgs a)
+{
+    constexpr int kRuns = T / kFan;
+    __shared__ double s_w[kRuns * (kFan + 1)];
+    const int R = rs_src(a), live = max(1, (R + T - 1) / T);
+    const int b = blockIdx.x, i0 = b * T, tid = threadIdx.x;
+    if (b >= live) return;  // block-uniform: past the source population
+    const int n = min(T, R - i0);
+    if (tid == 0 && i0 % rs_scan_size(R) == 0 && i0 / rs_scan_size(R) < rs_scan_blocks(R)) a.bcount[i0 / rs_scan_size(R)] = 0;
+    double w[1];
+    rs_block_weights<T, 1>(a, i0, n, (int)a.prev->emin_lo, w, s_w);
+    __syncthreads();  // the level table in s_w has been read
+    s_w[(tid / kFan) * (kFan + 1) + tid % kFan] = w[0];  // 0 past the population
+    __syncthreads();
+    if (tid < 32) {
+        const double tot = rs_run_sums(s_w + min(tid, kRuns - 1) * (kFan + 1), tid < kRuns ? kFan : 0);
+        if (tid < kRuns && tid * kFan < n) a.runP[b * kRuns + tid] = tot;
+    }
+    __syncthreads();
+    if (tid < n) a.P[i0 + tid] = s_w[(tid / kFan) * (kFan + 1) + tid % kFan];
+    if (last_block(a.sync, live)) rs_fused<T>(a, R);
+}
+
 __device__ __forceinline__ void rs_top_body(const ResampleArgs& a);
 // blocks of an instance that take part (block 0 always: it resets the copy
 // totals and S even of a population that died out)
@@ -260,10 +343,8 @@ __device__ __forceinline__ void rs_weights_launch(const ResampleArgs& a, int b)
     if (b >= live) return;  // block-uniform: past the source population
     rs_levels_body<T>(a, b, R, (int)a.prev->emin_lo);
     if (!last_block(a.sync, live)) return;
-    if (T == kWBlock) rs_fused(a, R);
-    else rs_top_body(a);  // levels >= 2 of the prefix
+    rs_top_body(a);  // levels >= 2 of the prefix
 }
-__global__ void __launch_bounds__(kWBlock) rs_weights_fused_kernel(ResampleArgs a) { rs_weights_launch<kWBlock>(a, blockIdx.x); }
 __global__ void __launch_bounds__(kWThreads) rs_weights_kernel(ResampleArgs a) { rs_weights_launch<kWThreads>(a, blockIdx.x); }
 __global__ void __launch_bounds__(kWThreads) rs_weights_batched(const ResampleArgs* tab)
 {
@@ -276,7 +357,7 @@ __global__ void __launch_bounds__(kWThreads) rs_weights_shard_kernel(ResampleArg
 }
 
 // Levels >= 2 of the prefix, by one block: bottom-up sums inside runs of the nb
-// block totals at up (each thread loads its run, then adds in order), then
+// block totals at up, then
 // top-down Q_{c-1} + l_j; up[0 .. nb) ends as the inclusive prefix.
 __device__ __forceinline__ void rs_top_levels(double* up, int nb)
 {
@@ -287,21 +368,10 @@ __device__ __forceinline__ void rs_top_levels(double* up, int nb)
     for (;;) {
         base[nl] = off; len[nl] = n; ++nl;
         const int nc = n <= kFan ? 1 : (n + kFan - 1) / kFan;
-        for (int c = tid; c < nc; c += nt) {
-            double* x = up + off + c * kFan;
-            const int cnt = min(kFan, n - c * kFan);
-            double acc = 0.0;
-            for (int j0 = 0; j0 < cnt; j0 += 8) {  // eight independent loads, then the additions
-                double v[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = j0 + j < cnt ? x[j0 + j] : 0.0;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = acc = __dadd_rn(acc, v[j]);  // +0 first and past the run: no change
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (j0 + j < cnt) x[j0 + j] = v[j];
-            }
-            if (n > kFan) up[off + n + c] = acc;
+        for (int c = tid; c - (tid & 31) < nc; c += nt) {  // by whole warps
+            const int cnt = c < nc ? min(kFan, n - c * kFan) : 0;
+            const double acc = rs_run_sums(up + off + (cnt ? c * kFan : 0), cnt);
+            if (c < nc && n > kFan) up[off + n + c] = acc;
         }
         __syncthreads();
         if (n <= kFan) break;  // one run left: its sums are the prefix of this level
@@ -472,13 +542,12 @@ __global__ void __launch_bounds__(32 * kRunWarps) rs_runs_batched(const Resample
 
 // Multinomial draws: the smallest i with x < P_i.  Each block stages the ends of
 // the segments of P (whole weights blocks) in shared memory and finds a draw's
-// segment there; the block's run table gives the run and the sums inside the run
-// the index, four ways at a time (three independent loads a round, three rounds
-// each, instead of ten dependent loads).  Copies are counted per replica and,
-// through shared memory, per scan block, so that the placement needs no pass
-// over the counts first.
+// segment there; the block's run table gives the run, four ways at a time (three
+// independent loads a round, three rounds, instead of five dependent loads), and
+// rs_first_near the index.  Copies are counted per replica and, through shared
+// memory, per scan block, so that the placement needs no pass over the counts
+// first.
 constexpr int kDrawThreads = 512;
-constexpr int kDrawSmall = 256;  // populations of at most kFuseR: more, smaller blocks
 constexpr int kMaxSeg = 2048;
 constexpr int kMaxHist = 1024;   // scan blocks counted in shared memory
 __device__ __forceinline__ int rs_seg_blocks(int nb)
@@ -518,6 +587,45 @@ __device__ __forceinline__ int rs_first_in_run(double q, long long x, int n, Pas
     int i = first_of_32([&](int j) { return j >= n || dbits(load(j)) >= t; });
     auto reached = [&](int j) { return past(dbits(__dadd_rn(q, load(j)))); };
     i = min(i, n - 1);
+    while (i > 0 && reached(i - 1)) --i;
+    while (i < n - 1 && !reached(i)) ++i;
+    return i;
+}
+// about the double's value, by integer work (only ever a guess)
+__device__ __forceinline__ float about(long long bits)
+{
+    return __int_as_float((int)max((bits >> 29) - (896ll << 23), 0ll));
+}
+// The same search for sums in global memory (l 32-byte aligned; readable up to
+// the next multiple of 32 bytes), four sums a load from where x would lie among
+// equal weights (next: the sum before the following run).  The lookups per lane
+// are what the search costs: two to four here, a dozen by three at a time.
+template <class Past>
+__device__ __forceinline__ int rs_first_near(const double* l, double q, double next, long long x, int n, Past past)
+{
+    const long long t = dbits(__dsub_rn(__longlong_as_double(x), q));
+    const float fq = about(dbits(q)), frac = (about(x) - fq) / (about(dbits(next)) - fq);
+    const int smax = (n - 1) >> 2;
+    int s = min(max((int)(frac * (kFan / 4)), 0), smax), i;
+    long long v0, v1, v2, v3;
+    bool left = false, right = false;
+    for (;;) {
+        asm("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(v0), "=l"(v1), "=l"(v2), "=l"(v3) : "l"(l + 4 * s));
+        if (s < smax && v3 < t) {  // past this quad
+            i = 4 * ++s;
+            if (left) break;
+            right = true;
+        } else if (s > 0 && !right && v0 >= t) {
+            --s;
+            left = true;
+        } else {
+            const int m = n - 4 * s;
+            i = 4 * s + (v0 < t) + (m > 1 && v1 < t) + (m > 2 && v2 < t) + (m > 3 && v3 < t);
+            break;
+        }
+    }
+    i = min(i, n - 1);
+    auto reached = [&](int j) { return past(dbits(__dadd_rn(q, l[j]))); };
     while (i > 0 && reached(i - 1)) --i;
     while (i < n - 1 && !reached(i)) ++i;
     return i;
@@ -563,9 +671,8 @@ __device__ __forceinline__ void rs_draws_body(const ResampleArgs& a, int q0, int
             return strict ? x < p : p >= x;
         });
         const int cc = min(c, leaves - 1), i0 = cc * kFan;
-        const int w = i0 + rs_first_in_run(a.runq[cc], x, min(kFan, R - i0),
-                                           [&](long long p) { return strict ? x < p : p >= x; },
-                                           [&](int t) { return a.P[i0 + t]; });
+        const int w = i0 + rs_first_near(a.P + i0, a.runq[cc], cc + 1 < leaves ? a.runq[cc + 1] : S, x, min(kFan, R - i0),
+                                         [&](long long p) { return strict ? x < p : p >= x; });
         atomicAdd(&a.counts[w], 1);
         if (hist) atomicAdd(&s_hist[w / sbits], 1);
         else atomicAdd(&a.bcount[w / sbits], 1);
@@ -618,6 +725,72 @@ __global__ void __launch_bounds__(kDrawThreads) rs_draws_shard_kernel(ResampleAr
 {
     rs_draws_shard_body(a, blockIdx.x * blockDim.x + threadIdx.x);
 }
+// Draws of a population of at most kFuseR: the whole run table in shared memory
+// (at most 64 KB), one block per SM, so that a draw makes only the gathers inside
+// its run.  Random gathers are what a draw costs: one L1 lookup per lane and load
+// (twenty a draw through global tables took half of the launch).  By ncu +-J
+// R = 10^5 10.3 -> 7.9 us, R = 5 x 10^4 8.3 -> 6.4 us.
+__global__ void __launch_bounds__(1024) rs_draws_fused_kernel(ResampleArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem_draws[];
+    static_assert(kFuseR <= kSmallScanR, "scan blocks of 1024");
+    __shared__ int s_hist[kFuseR / 1024];
+    const int R = a.R, tid = threadIdx.x, nt = blockDim.x;
+    const int nb = rs_wblocks(R), leaves = rs_leaves(R), ns = rs_scan_blocks(R);
+    long long* s_end = reinterpret_cast<long long*>(smem_draws);      // largest cumulative weight up to each run's end
+    double* s_q = reinterpret_cast<double*>(smem_draws) + leaves;     // sum before each run
+    for (int c = tid; c < leaves; c += nt) {
+        s_end[c] = max(dbits(a.bmax[nb + c / kFan]), dbits(a.runP[c]));
+        s_q[c] = a.runq[c];
+    }
+    if (tid < ns) s_hist[tid] = 0;
+    const double S = a.cur->S;
+    __syncthreads();
+    const int q = blockIdx.x * nt + tid;
+    if (q < a.Rn) {
+        const u32x4 o = philox((uint32_t)q, (uint32_t)a.k, 0u, a.c3, a.key0, a.key1);
+        const long long x = dbits(__dmul_rn(uniform53_int(o.x, o.y), S));  // x >= 0
+        const bool strict = x < s_end[leaves - 1];  // else x == S after rounding: the first P >= x
+        auto past = [&](long long p) { return strict ? x < p : p >= x; };
+        int lo = 0, hi = leaves - 1;  // the first run whose end is past x (the last one is)
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (past(s_end[mid])) hi = mid; else lo = mid + 1;
+        }
+        const int i0 = lo * kFan;
+        const int w = i0 + rs_first_near(a.P + i0, s_q[lo], lo + 1 < leaves ? s_q[lo + 1] : S, x, min(kFan, R - i0), past);
+        atomicAdd(&a.counts[w], 1);
+        atomicAdd(&s_hist[w / 1024], 1);
+    }
+    __syncthreads();
+    if (tid < ns && s_hist[tid]) atomicAdd(&a.bcount[tid], s_hist[tid]);
+}
+// dynamic shared memory of a kernel, asked for once per device (done: a bit each)
+template <class Kernel>
+static cudaError_t allow_smem(Kernel kern, int bytes, std::atomic<unsigned long long>& done)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || (dev < 64 && done.load(std::memory_order_acquire) >> dev & 1)) return e;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && dev < 64) done.fetch_or(1ull << dev, std::memory_order_release);
+    return e;
+}
+static cudaError_t launch_draws_fused(const ResampleArgs& a, cudaStream_t st)
+{
+    static std::atomic<unsigned long long> done{0};
+    const cudaError_t e = allow_smem(rs_draws_fused_kernel, 16 * rs_leaves(kFuseR), done);
+    if (e != cudaSuccess) return e;
+    // one block per SM where that gives it 128 to 1024 draws
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int t = ((a.Rn + sms - 1) / sms + 31) / 32 * 32;
+    t = t < 128 ? 128 : t > 1024 ? 1024 : t;
+    rs_draws_fused_kernel<<<(a.Rn + t - 1) / t, t, 16 * rs_leaves(a.R), st>>>(a);
+    return cudaGetLastError();
+}
+
 // two draws a thread in large populations: half the flushes of the copy totals
 constexpr int kDrawPer = 2;
 __global__ void __launch_bounds__(kDrawThreads) rs_draws_kernel(ResampleArgs a, int per)
@@ -812,7 +985,6 @@ __device__ __forceinline__ void rs_place_body(const ResampleArgs& a, int b, int 
         *a.Rdst = Rn;
         *a.Rdst_d = (double)Rn;
     }
-    if (b == 0 && tid == 1023) rs_lnq(a);
     for (int t = tid; t < total && off + t < cap; t += 1024) {
         int lo = 0, hi = SB - 1;  // the first replica whose inclusive sum exceeds t
         while (lo < hi) {
@@ -828,10 +1000,15 @@ __device__ __forceinline__ void rs_place_body(const ResampleArgs& a, int b, int 
 // of one cluster, a CTA per weights block.  The steps between which the larger
 // populations change launches are cluster barriers here (every CTA of a cluster
 // is resident, and the barrier's release and acquire order the global writes),
-// and every CTA completes the few values above its block by itself.  R = 1000:
-// 25 -> XX us.
+// and every CTA completes the few values above its block by itself.  Always eight
+// CTAs: the draws, FP64 operations of which an SM completes one warp's in 19
+// cycles, are shared out among them even if one block has all the weights.  By
+// ncu: R = 1000 18.6 us with one CTA, 14.5 us with eight (the launches of the larger
+// populations: 25 us); R = 4096 20.5 -> 18.4 us by the caller's clock.
 constexpr int kClusterCtas = 8;  // the portable cluster size
 constexpr int kClusterR = kClusterCtas * kWBlock;
+// staged, so that the draws' gathers stay off the L1 lookups: the sums inside the runs
+constexpr int cluster_smem(int R) { return (int)sizeof(double) * R; }
 __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -842,6 +1019,8 @@ __global__ void __launch_bounds__(kWBlock) rs_cluster_kernel(ResampleArgs a)
     __shared__ double s_up[kClusterCtas], s_rp[kRuns], s_rq[kRuns];
     __shared__ long long s_end[kClusterCtas];
     __shared__ int s_hist[kClusterCtas], s_min[32];
+    extern __shared__ __align__(16) unsigned char smem_cluster[];
+    double* s_P = reinterpret_cast<double*>(smem_cluster);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x, R = rs_src(a), nb = rs_wblocks(R), leaves = rs_leaves(R);
     int emin = 0;
@@ -865,13 +1044,9 @@ __global__ void __launch_bounds__(kWBlock) rs_cluster_kernel(ResampleArgs a)
     }
     if (b < rs_live_blocks(R)) rs_levels_body<kWBlock>(a, b, R, emin);
     cluster_sync();
-    if (tid == 0) {  // at most kFan block totals: one run of the next level
-        double acc = 0.0;
-        for (int t = 0; t < nb; ++t) {
-            const double v = __ldcg(a.upper + t);
-            acc = t == 0 ? v : __dadd_rn(acc, v);
-            s_up[t] = acc;
-        }
+    if (warp == 0) {  // at most kFan block totals: one run of the next level
+        const double up = rs_lane_sums<kClusterCtas>(lane < nb ? __ldcg(a.upper + lane) : 0.0);
+        if (lane < nb) s_up[lane] = up;
     }
     if (tid < kClusterCtas) s_hist[tid] = 0;
     __syncthreads();
@@ -884,16 +1059,18 @@ __global__ void __launch_bounds__(kWBlock) rs_cluster_kernel(ResampleArgs a)
         s_rp[t] = __ldcg(a.runP + t);
         s_rq[t] = __ldcg(a.runq + t);
     }
-    if (tid == 0) {
-        long long m = 0;
-        for (int t = 0; t < nb; ++t) {
-            m = max(m, dbits(__ldcg(a.bmax + t)));
-            s_end[t] = m;
-        }
-        if (b == 0) a.cur->S = __longlong_as_double(m);
+    if (a.scheme == 0)
+        for (int t = tid; t < R; t += kWBlock) s_P[t] = __ldcg(a.P + t);
+    if (warp == 0) {
+        long long m = lane < nb ? dbits(__ldcg(a.bmax + lane)) : 0;
+#pragma unroll
+        for (int o = 1; o < kClusterCtas; o <<= 1) m = max(m, __shfl_up_sync(0xffffffffu, m, o));
+        if (lane < nb) s_end[lane] = m;
+        if (b == kClusterCtas - 1 && lane == kClusterCtas - 1) a.cur->S = __longlong_as_double(m);
     }
     __syncthreads();
     const double S = nb > 0 ? __longlong_as_double(s_end[nb - 1]) : 0.0;
+    if (b == kClusterCtas - 1 && tid == kWBlock - 1) rs_lnq(a);  // rarely a warp with draws
     if (a.scheme == 1) {
         const int i = b * kWBlock + tid;
         int n = 0;
@@ -904,7 +1081,8 @@ __global__ void __launch_bounds__(kWBlock) rs_cluster_kernel(ResampleArgs a)
         n = __reduce_add_sync(0xffffffffu, n);
         if (lane == 0 && n) atomicAdd(&s_hist[b], n);
     } else {
-        for (int q = b * kWBlock + tid; q < a.Rn; q += gridDim.x * kWBlock) {
+        const int share = ((a.Rn + kClusterCtas - 1) / kClusterCtas + 31) / 32 * 32, end = min(a.Rn, (b + 1) * share);
+        for (int q = b * share + tid; q < end; q += kWBlock) {
             const u32x4 o = philox((uint32_t)q, (uint32_t)a.k, 0u, a.c3, a.key0, a.key1);
             const long long x = dbits(__dmul_rn(uniform53_int(o.x, o.y), S));  // x >= 0
             const bool strict = x < s_end[nb - 1];  // else x == S after rounding: the first P >= x
@@ -915,7 +1093,7 @@ __global__ void __launch_bounds__(kWBlock) rs_cluster_kernel(ResampleArgs a)
                 return bl * kFan + t >= leaves || past(dbits(s_rp[bl * kFan + t]));
             }));
             const int i = c * kFan + rs_first_in_run(s_rq[c], x, min(kFan, R - c * kFan), past,
-                                                     [&](int t) { return __ldcg(a.P + c * kFan + t); });
+                                                     [&](int t) { return s_P[c * kFan + t]; });
             atomicAdd(&a.counts[i], 1);
             atomicAdd(&s_hist[i / kWBlock], 1);
         }
@@ -928,6 +1106,10 @@ __global__ void __launch_bounds__(kWBlock) rs_cluster_kernel(ResampleArgs a)
 
 __device__ __forceinline__ void rs_place_launch(const ResampleArgs& a, int b)
 {
+    if (b == (int)gridDim.x - 1) {  // one more block than the placement needs: two FP64 logarithms
+        if (threadIdx.x == 0) rs_lnq(a);
+        return;
+    }
     const int R = rs_src(a);
     if (b >= max(1, rs_scan_blocks(R))) return;  // block-uniform
     if (rs_scan_size(R) == 1024) rs_place_body<1024>(a, b, R);
@@ -944,15 +1126,17 @@ cudaError_t launch_resample(const ResampleArgs& a, cudaStream_t st)
 {
     // a.R sizes the grids (the capacity when the population is in device memory)
     if (a.R <= kClusterR) {
-        int ctas = 1;
-        while (ctas < rs_wblocks(a.R)) ctas *= 2;
+        static std::atomic<unsigned long long> done{0};
+        const cudaError_t e = allow_smem(rs_cluster_kernel, cluster_smem(kClusterR), done);
+        if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = ctas;
+        cfg.gridDim = kClusterCtas;
         cfg.blockDim = kWBlock;
+        cfg.dynamicSmemBytes = cluster_smem(a.R);
         cfg.stream = st;
         cudaLaunchAttribute at = {};
         at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = ctas;
+        at.val.clusterDim.x = kClusterCtas;
         at.val.clusterDim.y = at.val.clusterDim.z = 1;
         cfg.attrs = &at;
         cfg.numAttrs = 1;
@@ -960,18 +1144,20 @@ cudaError_t launch_resample(const ResampleArgs& a, cudaStream_t st)
     }
     const bool fused = a.R <= kFuseR;
     if (fused) {
-        rs_weights_fused_kernel<<<rs_wblocks(a.R), kWBlock, 0, st>>>(a);
+        if (a.kind == 0) rs_weights_fused_kernel<1024><<<(a.R + 1023) / 1024, 1024, 0, st>>>(a);
+        else rs_weights_fused_kernel<256><<<(a.R + 255) / 256, 256, 0, st>>>(a);
     } else {
         rs_weights_kernel<<<rs_wblocks(a.R), kWThreads, 0, st>>>(a);
         rs_runs_kernel<<<(rs_wblocks(a.R) + kRunWarps - 1) / kRunWarps, 32 * kRunWarps, 0, st>>>(a);
     }
     if (a.scheme == 1)
         rs_nearest_kernel<<<(a.R + 255) / 256, 256, 0, st>>>(a);
-    else if (fused)
-        rs_draws_kernel<<<(a.Rn + kDrawSmall - 1) / kDrawSmall, kDrawSmall, 0, st>>>(a, 1);
-    else
+    else if (fused) {
+        const cudaError_t e = launch_draws_fused(a, st);
+        if (e != cudaSuccess) return e;
+    } else
         rs_draws_kernel<<<(a.Rn + kDrawPer * kDrawThreads - 1) / (kDrawPer * kDrawThreads), kDrawThreads, 0, st>>>(a, kDrawPer);
-    rs_place_kernel<<<place_grid(a.R), 1024, 0, st>>>(a);
+    rs_place_kernel<<<place_grid(a.R) + 1, 1024, 0, st>>>(a);
     return cudaGetLastError();
 }
 int resample_launches(const ResampleArgs& a) { return a.R <= kClusterR ? 1 : a.R <= kFuseR ? 3 : 4; }
@@ -1009,7 +1195,7 @@ cudaError_t launch_resample_batched(const ResampleArgs* tab, int n_inst, int max
     rs_weights_batched<<<dim3(rs_wblocks(maxR), ni), kWThreads, 0, st>>>(tab);
     rs_runs_batched<<<dim3((rs_wblocks(maxR) + kRunWarps - 1) / kRunWarps, ni), 32 * kRunWarps, 0, st>>>(tab);
     rs_draws_batched<<<dim3((maxR + kDrawThreads - 1) / kDrawThreads, ni), kDrawThreads, 0, st>>>(tab);
-    rs_place_batched<<<dim3(place_grid(maxR), ni), 1024, 0, st>>>(tab);
+    rs_place_batched<<<dim3(place_grid(maxR) + 1, ni), 1024, 0, st>>>(tab);
     return cudaGetLastError();
 }
 
@@ -1035,8 +1221,8 @@ cudaError_t launch_logc_table(double* t, cudaStream_t st)
 // GPU.  The launch is latency: one round of loads, then short chains.  A run of
 // equal family ids ends at the next start, found from the warp's ballot, the
 // other warps' first starts, and only for the last run of a window by a search
-// beyond it (the whole warp, 32 probes a round).  R = 10^5: 15 -> XX us, 5 x 10^4
-// with real couplings 17 -> XX us (small blocks: the FP64 sums spread over the
+// beyond it (the whole warp, 32 probes a round).  R = 10^5: 15.6 -> 10.1 us, 5 x 10^4
+// with real couplings 17.2 -> 11.2 us (small blocks: the FP64 sums spread over the
 // SMs).
 constexpr int kObsThreads = 256;
 constexpr int kObsWarps = kObsThreads / 32;

@@ -92,3 +92,21 @@ def test_long_families(pa, oracle, R, beta):
         assert pop.observables(2)["S_f"] == pytest.approx(np.log(R) - (c * np.log(c)).sum() / R, abs=1e-8)
     finally:
         pop.close()
+
+
+@pytest.mark.parametrize("R", [33, 1000, 8193, 33_025, 131_072, 131_073])
+def test_real_population_resample_sizes(pa, oracle, R):
+    """Real couplings: 256-replica weights blocks up to 131072 replicas
+    (ln Q as test_gpu_fullsize compares it)."""
+    P, O = pa, oracle
+    J, betas, seed = W.couplings_gauss(2, 2, 5), np.array([0.0, 0.4, 2.1]), 7 + R
+    pop = P.Population(2, 2, P.PA_REAL, J, None, R, betas, 1, seed)
+    try:
+        assert pop.step()
+        for k in (1, 2):
+            want = O.resample(1, _pairs(P.pa_get_energies(pop.ctx, 1), 1), betas[k - 1], betas[k], k, seed)
+            assert pop.step()
+            np.testing.assert_array_equal(P.pa_get_parents(pop.ctx), want["parent"])
+            assert pop.observables(k)["lnQ"] == pytest.approx(want["lnQ"], rel=1e-10, abs=1e-10)
+    finally:
+        pop.close()
