@@ -163,8 +163,9 @@ int pa_create_ws(pa_ctx** out, int D, int L, int kind, const float* J, const flo
  * beta_{k-1} (k > 0), N_S sweeps at beta_k, energies and observables.
  * Asynchronous on the context's stream.  PA_EDONE after the last temperature. */
 int pa_anneal_step(pa_ctx* ctx);
-/* n_steps steps (-1: the rest of the schedule) captured once into a CUDA graph
- * and replayed; identical results to repeated pa_anneal_step. */
+/* n_steps steps (-1: the rest of the schedule): the first ones enqueued one by
+ * one, the others captured into a CUDA graph meanwhile and launched behind them;
+ * identical results to repeated pa_anneal_step. */
 int pa_anneal(pa_ctx* ctx, int n_steps);
 int pa_current_step(const pa_ctx* ctx);
 int pa_synchronize(pa_ctx* ctx);
