@@ -27,7 +27,8 @@
 // dE = 2 S_i f (exact), x = f32(beta) dE; accept iff x <= 0 or
 // r < floor(spec_expf(-x) 2^32), decided through a device-verified guard band
 // around that threshold (same decisions; see accept_band).  Energies are
-// exact int128 sums of J * 2^96.
+// exact int128 sums of J * 2^96.  Only the lattices whose threshold tables do not
+// fit (pa_real_table.cuh) take this tile.
 #pragma once
 #include <type_traits>
 #include "pa_device.cuh"
@@ -66,13 +67,20 @@ __device__ __forceinline__ uint64_t rep32(uint32_t v) { return ((uint64_t)v << 3
 // threshold's bit for each lane's class) is selected by the count bits:
 // n = 0 -> v00, n = 1 -> v01, n = 2 -> v10 (0 / ~0 masks of this plane).
 // A lane whose plane bit differs from T is decided: accepted if T = 1.
+// LAST: acc takes ~pl in every lane still compared instead, so that a decided
+// lane keeps the plane that decided it (it differed from T: accepted if it is 0),
+// four LOP3 a half plane instead of five; the caller clears the lanes left in U.
+// Only where no plane has all threshold bits 0 from the start (L=16, R=10^6, mean
+// launch of k < 25: 13.24 -> 13.08 ms); such planes would take two LOP3 instead of
+// one (whole schedule at L=16, R=10^5: 1275 -> 1302 us a launch).
+template <bool LAST = false>
 __device__ __forceinline__ void plane_step(uint64_t pl, uint32_t v00, uint32_t v01, uint32_t v10,
                                            uint64_t b0, uint64_t b1, uint64_t& U, uint64_t& acc)
 {
     const uint64_t V00 = rep32(v00), V01 = rep32(v01), V10 = rep32(v10);
     const uint64_t inner = (b0 & V01) | (~b0 & V00);
     const uint64_t T = (b1 & V10) | (~b1 & inner);
-    acc |= U & T & ~pl;
+    acc = LAST ? (U & ~pl) | (~U & acc) : acc | (U & T & ~pl);
     U &= ~(T ^ pl);
 }
 
@@ -394,11 +402,12 @@ __device__ __forceinline__ void sweep_packed_tile(const PackedStep& s, const Pac
         } else {
             // high temperature: threshold bits of 1 from the first planes on
             run_calls([&](int m, const u32x4& o) {
-                plane_step((uint64_t)o.x | ((uint64_t)o.y << 32), s.v00[2 * m], s.v01[2 * m],
+                plane_step<true>((uint64_t)o.x | ((uint64_t)o.y << 32), s.v00[2 * m], s.v01[2 * m],
                            s.v10[2 * m], b0, b1, U, acc);
-                plane_step((uint64_t)o.z | ((uint64_t)o.w << 32), s.v00[2 * m + 1], s.v01[2 * m + 1],
+                plane_step<true>((uint64_t)o.z | ((uint64_t)o.w << 32), s.v00[2 * m + 1], s.v01[2 * m + 1],
                            s.v10[2 * m + 1], b0, b1, U, acc);
             });
+            acc &= ~U;
         }
     };
     // lanes that flip without a comparison (acc) and lanes that need one (U)
