@@ -45,10 +45,10 @@ UNIT = "attempts/ns"
 # sweep (packed: 1 bit each way; int8: 1 byte each way)
 BYTES_PER_ATTEMPT = {"packed": 0.25, "i8": 2.0}
 # streaming bytes per resampled replica (the replica gather is fused into the
-# sweep): energy read 4 (+-J; 16 for int128), weight write 8, local prefix
-# write 8, prefix finalize read + write 16, copy-count atomic 8, block sums
-# read 4, fill: counts read + clear 8, parent write 4, family read + write 8
-RESAMPLE_BYTES_PER_REPLICA = {0: 68, 1: 80}
+# sweep): energy read 4 (+-J; 16 for int128), the sums inside the runs written
+# and read by the draws 16, copy-count atomic 8, placement: counts read + clear
+# 8, parent write 4, family read + write 8
+RESAMPLE_BYTES_PER_REPLICA = {0: 48, 1: 60}
 
 
 def _peaks():
@@ -318,7 +318,7 @@ def run_gpu(args, wl_name):
                                "frac": RESAMPLE_BYTES_PER_REPLICA[kind] * R / (rs_ms * 1e-3) / 1e9 / peak,
                                "bytes_per_replica": RESAMPLE_BYTES_PER_REPLICA[kind],
                                "note": "all resampling launches of a step; latency-bound by the fixed-order "
-                                       "sequential FP64 prefix and the binary-search draws"}
+                                       "sequential FP64 prefix and the draws' random gathers"}
                               if rs_ms > 0 else None),
         "gpu_launches": int(launches1 - launches0),
         "clocks": clocks,

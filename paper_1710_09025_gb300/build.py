@@ -19,7 +19,7 @@ LIB = os.path.join(BUILD, "libpamc.so")
 SOURCES = ["pa_packed_part0.cu", "pa_packed_part1.cu", "pa_packed_part2.cu", "pa_packed_part3.cu",
            "pa_batch.cu", "pa_real.cu", "pa_real_table_plain.cu", "pa_real_table_field.cu", "pa_api.cu", "pa_packed.cu", "pa_resample.cu", "pa_noalloc.cu",
            "pa_icm.cu", "pa_gather_grad.cu"]
-HEADERS = ["pa_device.cuh", "pa_internal.h", "pa_sweep_tiles.cuh", "pa_packed_sweep.cuh", "pa_real_table.cuh"]
+HEADERS = ["pa_device.cuh", "pa_internal.h", "pa_launch.h", "pa_sweep_tiles.cuh", "pa_packed_sweep.cuh", "pa_real_table.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-ffp-contract=off",
          "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]

@@ -76,7 +76,7 @@ struct pa_ctx {
     unsigned long long* hist;
     double *gbar_d, *dJ_d, *dh_d;
     pa::ObsPartial* obspart;
-    double* logc;               // log(c) table of the family entropy
+    double* logc;               // c ln c table of the family entropy
     double* Rk_d;               // populations as doubles (gradient normalisation)
     cudaGraphExec_t gexec;
     std::string err;
@@ -1547,7 +1547,7 @@ extern "C" void pa_destroy(pa_ctx* c)
 // (built by plan_step, so the batched launches and the per-instance launches
 // follow the same ping-pong sequence).  A batched step is: k = 0 initialisation
 // per instance; resampling for all instances (one launch per kernel); one
-// persistent sweep launch over a work queue of (instance, tile) items; the
+// or two persistent sweep launches over work queues of (instance, tile) items; the
 // observables for all instances.
 
 #include <algorithm>

@@ -1,5 +1,6 @@
-// pa_batch.cu -- the batched sweep: one persistent launch over the replica
-// tiles of many instances (mixed L, +-J and real couplings).
+// pa_batch.cu -- the batched sweep: persistent launches over the replica tiles of
+// many instances (mixed L, +-J and real couplings): one for the packed tiles (and
+// the real couplings without threshold tables), one beside it for the tables.
 //
 // Blocks take work items (instance, tile) from a queue in global memory (one
 // atomic counter per temperature) and run the same tile functions as the

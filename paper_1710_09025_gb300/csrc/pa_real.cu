@@ -1,4 +1,6 @@
-// pa_real.cu -- real (Gaussian) couplings: int8 spins, FP32 local fields.
+// pa_real.cu -- real (Gaussian) couplings: int8 spins, FP32 local fields.  The
+// dispatch, the check of the guard band and the per-attempt kernel of the lattices
+// whose threshold tables do not fit (pa_real_table.cuh has the others).
 //
 // Sec. II.B Metropolis sweeps (checkerboard order of Sec. III.A) for
 // H = -sum J_ij S_i S_j - sum h_i S_i with FP32 couplings (Sec. II.A draws

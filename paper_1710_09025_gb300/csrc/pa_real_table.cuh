@@ -37,6 +37,7 @@
 #pragma once
 #include "pa_device.cuh"
 #include "pa_internal.h"
+#include "pa_launch.h"
 #include "pa_sweep_tiles.cuh"
 
 namespace pa {
@@ -675,12 +676,9 @@ static cudaError_t launch_real_table(const RealSweepArgs& a, cudaStream_t st)
 {
     using SH = TabShape<D, L, FIELD>;
     auto kern = sweep_real_table_kernel<D, L, FIELD>;
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM_GRAD);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static std::atomic<unsigned long long> done{0};
+    const cudaError_t e = allow_smem(kern, (int)SH::SMEM_GRAD, done);
+    if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per = 0;
     const size_t smem = a.i.cJ ? SH::SMEM_GRAD : SH::SMEM;
     cudaGetDevice(&dev);

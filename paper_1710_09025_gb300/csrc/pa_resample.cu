@@ -18,8 +18,7 @@
 // stay contiguous (Sec. V.A).
 #include "pa_device.cuh"
 #include "pa_internal.h"
-
-#include <atomic>
+#include "pa_launch.h"
 
 namespace pa {
 
@@ -764,17 +763,6 @@ __global__ void __launch_bounds__(1024) rs_draws_fused_kernel(ResampleArgs a)
     }
     __syncthreads();
     if (tid < ns && s_hist[tid]) atomicAdd(&a.bcount[tid], s_hist[tid]);
-}
-// dynamic shared memory of a kernel, asked for once per device (done: a bit each)
-template <class Kernel>
-static cudaError_t allow_smem(Kernel kern, int bytes, std::atomic<unsigned long long>& done)
-{
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess || (dev < 64 && done.load(std::memory_order_acquire) >> dev & 1)) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess && dev < 64) done.fetch_or(1ull << dev, std::memory_order_release);
-    return e;
 }
 static cudaError_t launch_draws_fused(const ResampleArgs& a, cudaStream_t st)
 {

@@ -70,8 +70,8 @@ def run_partitioned(descs: Sequence[dict], run_instances: Callable, n_temps: int
 
 
 def gpu_batch_runner(P, D, betas, n_sweeps, seed, stream=None):
-    """run_instances for the CUDA library: one batch (one persistent sweep
-    launch per step, graph-captured) of the given instances, instance id =
+    """run_instances for the CUDA library: one batch (persistent sweep
+    launches per step, graph-captured) of the given instances, instance id =
     global index; returns (beta F_k, <E>_k) per instance."""
     def run(descs, ids):
         if not descs:

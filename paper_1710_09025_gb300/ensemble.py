@@ -20,7 +20,7 @@ from . import schedules as S
 
 def betaF_seed_batch(P, D, L, kind, J, h, R, betas, n_sweeps, seed, n_runs, stream=None):
     """beta F_k (n_runs x n_temps) of n_runs independent runs of one instance,
-    run as one batch (one persistent sweep launch per step, graph-captured)."""
+    run as one batch (persistent sweep launches per step, graph-captured)."""
     if n_runs < 2:
         raise ValueError("need at least two runs")
     descs = [dict(L=L, kind=kind, J=J, h=h, R=R, rng_instance=m) for m in range(n_runs)]
