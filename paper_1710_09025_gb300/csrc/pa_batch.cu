@@ -10,6 +10,8 @@
 #include "pa_real_table.cuh"
 #include "pa_sweep_tiles.cuh"
 
+#include <algorithm>
+
 namespace pa {
 
 constexpr int kBatchThreads = 256;
@@ -141,10 +143,25 @@ bool batch_class(int D, int L, int kind, bool field, int mult, int chunk, int G,
     return false;
 }
 
+// Shared memory of the largest item of each launch.  The limit belongs to the
+// kernel on a device, not to a batch: it is raised to this once and never set to
+// what one batch needs, which would refuse the launches of another batch with
+// larger items.
+#define XP(idx, l)                                                          \
+    PackedShape<3, l, default_shape<3, l>().gpb, kBatchThreads, false>::SMEM, \
+        PackedShape<3, l, 2 * default_shape<3, l>().gpb, kBatchThreads, false>::SMEM,
+#define XR(idx, l) RealShape<3, l, kBatchThreads / 32>::SMEM,
+#define XT(idx, l, f) TabShape<3, l, f>::SMEM,
+constexpr size_t kBatchSmem = std::max({PA_BATCH_PACKED(XP) PA_BATCH_REAL(XR) size_t(0)});
+constexpr size_t kBatchTableSmem = std::max({PA_BATCH_TABLE(XT) size_t(0)});
+#undef XP
+#undef XR
+#undef XT
+
 cudaError_t batch_sweep_occupancy(size_t smem, int* blocks_per_sm)
 {
-    cudaError_t e = cudaFuncSetAttribute(sweep_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    static std::atomic<unsigned long long> done{0};
+    const cudaError_t e = allow_smem(sweep_batch_kernel, (int)kBatchSmem, done);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, sweep_batch_kernel,
                                                          kBatchThreads, smem);
@@ -160,8 +177,8 @@ cudaError_t launch_sweep_batched(const PackedStep& ps, const RealStep& rs, const
 
 cudaError_t batch_table_occupancy(size_t smem, int* blocks_per_sm)
 {
-    cudaError_t e = cudaFuncSetAttribute(sweep_batch_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    static std::atomic<unsigned long long> done{0};
+    const cudaError_t e = allow_smem(sweep_batch_table_kernel, (int)kBatchTableSmem, done);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, sweep_batch_table_kernel, kTabThreads, smem);
 }

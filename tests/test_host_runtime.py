@@ -1,0 +1,98 @@
+"""The library's host code against a CUDA runtime without a device
+(shims/fake_cudart.cpp): the library's own objects, linked against a runtime that
+records calls, keeps each kernel's shared-memory limit per device and refuses
+the launches above it, and fails the call that a test names.  Kernels do not
+run; what they compute is covered on the GPU."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+STREAM = 0x4000  # a handle that the fake runtime takes for a stream
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    from paper_1710_09025_gb300 import build as B
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    B.build()
+    objs = [os.path.join(B.BUILD, s.replace(".cu", ".o")) for s in B.SOURCES]
+    out = tmp_path_factory.mktemp("fake") / "libpamc_fake.so"
+    subprocess.run(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", "-Wl,-Bsymbolic",
+                    "-I" + os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include"),
+                    os.path.join(ROOT, "tests", "shims", "fake_cudart.cpp"), *objs, "-o", str(out)], check=True)
+    return str(out)
+
+
+class Fake:
+    def __init__(self, lib):
+        lib.fake_log.restype = ctypes.c_char_p
+        lib.fake_fail.argtypes = [ctypes.c_char_p, ctypes.c_int]
+        self.lib = lib
+
+    def reset(self):
+        self.lib.fake_reset()
+        self.lib.fake_device(0)
+
+    def device(self, d):
+        self.lib.fake_device(d)
+
+    def fail(self, name, after=0):
+        self.lib.fake_fail(name.encode(), after)
+
+    def log(self):
+        return self.lib.fake_log().decode().splitlines()
+
+    def launched(self, kernel):
+        return [x for x in self.log() if x.startswith("launch ") and kernel in x]
+
+
+@pytest.fixture
+def fake(fake_lib, monkeypatch):
+    """(the package bound to the library on the fake runtime, its controls)"""
+    import paper_1710_09025_gb300 as P
+    monkeypatch.setattr(P, "_lib", None)
+    f = Fake(P.load(fake_lib))
+    f.reset()
+    yield P, f
+    f.reset()
+
+
+def _couplings(kind, L, seed=1):
+    from paper_1710_09025_gb300 import workloads as W
+    return W.couplings_gauss(3, L, seed) if kind else W.couplings_pm(3, L, seed)
+
+
+def _batch(P, insts, n=4, sweeps=2, **opts):
+    """insts: (kind, L, R, with a field)"""
+    from paper_1710_09025_gb300 import workloads as W
+    descs = [dict(L=L, kind=kind, J=_couplings(kind, L, i), h=W.field_uniform(L ** 3, i) if field else None, R=R,
+                  rng_instance=i) for i, (kind, L, R, field) in enumerate(insts)]
+    return P.pa_batch_create(3, descs, np.linspace(0.0, 1.0, n), sweeps, 7, P.pa_options_default(**opts), STREAM)
+
+
+@pytest.mark.parametrize("first,second", [
+    ([(1, 10, 200, False)], [(1, 4, 200, False)]),                            # table launch: about 200 KB, then 70
+    ([(0, 16, 200, False)], [(1, 4, 200, False)]),                            # mixed launch: no such item in the second
+    ([(1, 12, 200, False), (1, 10, 200, False)], [(0, 4, 200, False), (1, 6, 200, True)]),
+    ([(0, 16, 200, False)], [(0, 4, 200, False)]),
+])
+@pytest.mark.parametrize("tune", [0, -1])
+def test_a_batch_leaves_another_batchs_launches_alone(fake, first, second, tune):
+    P, f = fake
+    a = _batch(P, first, threads=tune)
+    b = _batch(P, second, threads=tune)
+    try:
+        for x in (a, b):
+            P.pa_batch_run(x, 2)
+            assert P.pa_batch_step(x) and P.pa_batch_step(x)
+            assert P.pa_batch_current_step(x) == 4
+    finally:
+        P.pa_batch_destroy(a)
+        P.pa_batch_destroy(b)
