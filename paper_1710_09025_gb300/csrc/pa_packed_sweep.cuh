@@ -3,6 +3,7 @@
 // block choices, packed or int8 storage); the sizes are spread over the
 // translation units pa_packed_part0..3.cu so that they compile in parallel.
 #pragma once
+#include "pa_launch.h"
 #include "pa_sweep_tiles.cuh"
 
 namespace pa {
@@ -63,12 +64,9 @@ static cudaError_t launch_one(const PackedSweepArgs& a, int grid, int spread, cu
 {
     const size_t smem = PackedShape<D, L, GPB, THREADS>::SMEM;
     auto kern = sweep_packed_kernel<D, L, GPB, THREADS, I8, SHARD>;
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static std::atomic<unsigned long long> done{0};
+    const cudaError_t e = allow_smem(kern, (int)smem, done);
+    if (e != cudaSuccess) return e;
     kern<<<grid, THREADS, smem, st>>>(a, spread);
     return cudaGetLastError();
 }

@@ -116,13 +116,9 @@ static cudaError_t launch_real_one(const RealSweepArgs& a, int grid, cudaStream_
 {
     const size_t smem = a.i.cJ ? RealShape<D, L, WARPS>::SMEM_GRAD : RealShape<D, L, WARPS>::SMEM;
     auto kern = sweep_real_kernel<D, L, WARPS>;
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)RealShape<D, L, WARPS>::SMEM_GRAD);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static std::atomic<unsigned long long> done{0};
+    const cudaError_t e = allow_smem(kern, (int)RealShape<D, L, WARPS>::SMEM_GRAD, done);
+    if (e != cudaSuccess) return e;
     if (grid <= 0) {
         int dev = 0, sms = 0, per = 0;
         cudaGetDevice(&dev);

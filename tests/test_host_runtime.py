@@ -96,3 +96,22 @@ def test_a_batch_leaves_another_batchs_launches_alone(fake, first, second, tune)
     finally:
         P.pa_batch_destroy(a)
         P.pa_batch_destroy(b)
+
+
+@pytest.mark.parametrize("kind,L,field,opts", [
+    (0, 16, False, {}), (0, 16, False, dict(layout=2)), (0, 16, False, dict(groups_per_block=2)), (0, 10, False, {}),
+    (1, 12, False, {}), (1, 12, True, dict(accumulate_grad=1)), (1, 10, True, dict(threads=128)), (1, 10, False, {}),
+    (1, 8, True, {}),
+])
+def test_every_device_gets_the_shared_memory_limit(fake, kind, L, field, opts):
+    """Tiles above 48 KB: the limit is asked for on each device that launches them."""
+    from paper_1710_09025_gb300 import workloads as W
+    P, f = fake
+    for dev in (0, 1, 2, 0):
+        f.device(dev)
+        h = W.field_uniform(L ** 3, 3) if field else None
+        ctx = P.pa_create(3, L, kind, _couplings(kind, L), h, 9000, [0.0, 0.5], 1, 5, P.pa_options_default(**opts), STREAM)
+        try:
+            assert P.pa_anneal_step(ctx) and P.pa_anneal_step(ctx)
+        finally:
+            P.pa_destroy(ctx)
