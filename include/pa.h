@@ -164,7 +164,8 @@ int pa_create_ws(pa_ctx** out, int D, int L, int kind, const float* J, const flo
  * Asynchronous on the context's stream.  PA_EDONE after the last temperature. */
 int pa_anneal_step(pa_ctx* ctx);
 /* n_steps steps (-1: the rest of the schedule): the first ones enqueued one by
- * one, the others captured into a CUDA graph meanwhile and launched behind them;
+ * one, the others captured into a CUDA graph meanwhile and launched behind them
+ * (or enqueued one by one as well, should the capture or the graph fail);
  * identical results to repeated pa_anneal_step. */
 int pa_anneal(pa_ctx* ctx, int n_steps);
 int pa_current_step(const pa_ctx* ctx);

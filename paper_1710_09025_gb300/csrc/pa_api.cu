@@ -909,6 +909,40 @@ static int steps_ahead(const pa_ctx* c, int n)
     return std::min(n, (int)std::ceil(n * b / (t + b)));
 }
 
+// n steps captured into one graph and launched; after an error the context is
+// where it was and nothing of them runs
+static int anneal_graph(pa_ctx* c, int n)
+{
+    const int k_save = c->k_next, cur_save = c->cur, fam_save = c->famcur;
+    const long long launches_save = c->launches;
+    const char* what = "stream capture: ";
+    cudaGraph_t g = nullptr;
+    int rc = PA_OK;
+    cudaError_t e = cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        c->capturing = true;
+        for (int t = 0; t < n && rc == PA_OK; ++t) rc = enqueue_step(c);
+        c->capturing = false;
+        e = cudaStreamEndCapture(c->st, &g);
+    }
+    if (rc == PA_OK && e == cudaSuccess) {
+        what = "cudaGraphInstantiate: ";
+        e = cudaGraphInstantiate(&c->gexec, g, 0);
+        if (e != cudaSuccess) c->gexec = nullptr;
+    }
+    if (g) cudaGraphDestroy(g);
+    if (rc == PA_OK && e == cudaSuccess) {
+        what = "cudaGraphLaunch: ";
+        e = cudaGraphLaunch(c->gexec, c->st);
+    }
+    if (rc == PA_OK && e == cudaSuccess) return PA_OK;
+    cudaGetLastError();  // reported here: the next launch's check must not find it
+    c->launches = launches_save;
+    c->k_next = k_save; c->cur = cur_save; c->famcur = fam_save;
+    if (rc == PA_OK) { c->err = std::string(what) + cudaGetErrorString(e); rc = PA_ECUDA; }
+    return rc;
+}
+
 extern "C" int pa_anneal(pa_ctx* c, int n_steps)
 {
     if (!c) return PA_EINVAL;
@@ -932,37 +966,20 @@ extern "C" int pa_anneal(pa_ctx* c, int n_steps)
     int rc = PA_OK, ahead = steps_ahead(c, n);
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (ahead > 0) PA_CK(c, cudaStreamIsCapturing(c->st, &cs));
-    if (ahead > 0 && cs == cudaStreamCaptureStatusNone) {
+    if (ahead == 0 || cs != cudaStreamCaptureStatusNone) return anneal_graph(c, n);
+    auto eager = [&](int steps) {
         c->capturing = true;  // no phase events
-        for (; ahead > 0 && rc == PA_OK; --ahead, --n) rc = enqueue_step(c);
+        for (; steps > 0 && rc == PA_OK; --steps, --n) rc = enqueue_step(c);
         c->capturing = false;
-        if (rc != PA_OK || n == 0) return rc;
-    }
-    const int k_save = c->k_next, cur_save = c->cur, fam_save = c->famcur;
-    const long long launches_save = c->launches;
-    PA_CK(c, cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal));
-    c->capturing = true;
-    for (int t = 0; t < n && rc == PA_OK; ++t) rc = enqueue_step(c);
-    c->capturing = false;
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamEndCapture(c->st, &g);
-    if (rc != PA_OK || e != cudaSuccess) c->launches = launches_save;
-    if (rc != PA_OK || e != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        c->k_next = k_save; c->cur = cur_save; c->famcur = fam_save;
-        if (rc == PA_OK) { c->err = std::string("stream capture: ") + cudaGetErrorString(e); rc = PA_ECUDA; }
         return rc;
-    }
-    e = cudaGraphInstantiate(&c->gexec, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) {
-        c->k_next = k_save; c->cur = cur_save; c->famcur = fam_save;
-        c->gexec = nullptr;
-        c->err = std::string("cudaGraphInstantiate: ") + cudaGetErrorString(e);
-        return PA_ECUDA;
-    }
-    PA_CK(c, cudaGraphLaunch(c->gexec, c->st));
-    return PA_OK;
+    };
+    if (eager(ahead) != PA_OK || n == 0) return rc;
+    const std::string err = c->err;
+    if (anneal_graph(c, n) == PA_OK) return PA_OK;
+    // no graph, with steps enqueued already: the others follow them one by one, so
+    // that the call still makes the steps that it was asked for
+    c->err = err;
+    return eager(n);
 }
 
 extern "C" int pa_current_step(const pa_ctx* c) { return c ? c->k_next : PA_EINVAL; }

@@ -115,3 +115,54 @@ def test_every_device_gets_the_shared_memory_limit(fake, kind, L, field, opts):
             assert P.pa_anneal_step(ctx) and P.pa_anneal_step(ctx)
         finally:
             P.pa_destroy(ctx)
+
+
+def _kernels(log):
+    return [x for x in log if x.startswith("launch ")]
+
+
+@pytest.mark.parametrize("call,after", [("cudaStreamBeginCapture", 0), ("cudaStreamEndCapture", 0),
+                                        ("cudaGraphInstantiate", 0), ("cudaGraphLaunch", 0), ("observe_kernel", 40)])
+@pytest.mark.parametrize("n", [-1, 50])
+def test_an_anneal_makes_its_steps_without_a_graph(fake, call, after, n):
+    """pa_anneal enqueues its first steps before it captures the others.  When the
+    graph cannot be had it still makes exactly the steps it was asked for, each
+    once and in order, and can be called again."""
+    P, f = fake
+    args = (3, 4, 0, _couplings(0, 4), None, 10_000, np.linspace(0.0, 1.0, 61), 10, 5)
+    want = P.pa_create(*args, stream=STREAM)
+    got = P.pa_create(*args, stream=STREAM)
+    try:
+        f.reset()
+        for _ in range(61):
+            assert P.pa_anneal_step(want)
+        steps = _kernels(f.log())
+        f.reset()
+        f.fail(call, after)
+        P.pa_anneal(got, n)
+        assert P.pa_current_step(got) == (61 if n < 0 else n)
+        if n > 0:
+            P.pa_anneal(got, 61 - n)
+        assert _kernels(f.log()) == steps
+    finally:
+        P.pa_destroy(want)
+        P.pa_destroy(got)
+
+
+@pytest.mark.parametrize("call,after", [("cudaStreamBeginCapture", 0), ("cudaGraphInstantiate", 0),
+                                        ("cudaGraphLaunch", 0), ("observe_kernel", 3)])
+def test_an_anneal_without_eager_steps_is_all_or_nothing(fake, call, after):
+    """On the legacy stream nothing runs before the graph: an error leaves the
+    context where it was."""
+    P, f = fake
+    ctx = P.pa_create(3, 4, 0, _couplings(0, 4), None, 10_000, np.linspace(0.0, 1.0, 9), 10, 5, stream=1)
+    try:
+        f.reset()
+        f.fail(call, after)
+        with pytest.raises(P.PAError):
+            P.pa_anneal(ctx)
+        assert P.pa_current_step(ctx) == 0 and not _kernels(f.log())
+        P.pa_anneal(ctx)
+        assert P.pa_current_step(ctx) == 9 and len(f.launched("observe_kernel")) == 9
+    finally:
+        P.pa_destroy(ctx)
