@@ -1757,6 +1757,7 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
     // work items, most expensive first (estimated thread-instructions per
     // tile): one list for the launch of each groups-per-block multiplier, one
     // (m = 0) for the threshold-table launch
+    std::map<int, int> tuned_items;
     for (int m = 0; m <= 2 && e == cudaSuccess; ++m) {
         struct It { double cost; int inst, tile; };
         std::vector<It> items;
@@ -1767,6 +1768,7 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
             size_t sm;
             pa::batch_class(D, c->L, c->kind, c->field != 0, m > 0 ? m : 1, b->tchunk, c->G, c->R, &cls, &tiles, &sm);
             if ((cls >= pa::kBatchTableBase) != (m == 0)) continue;
+            if (m == 1) tuned_items[cls] += tiles;
             smax = std::max(smax, sm);
             int gpb = 0, thr = 0;
             pa::packed_default_shape(D, c->L, &gpb, &thr);
@@ -1820,13 +1822,10 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
         }
     }
     if (b->n_items[0] == 0) b->tuned = true;  // nothing to tune
-    // signature of the batch for the tuning cache: SM count and class histogram
-    std::map<std::pair<int, int>, int> hist;
-    for (auto* c : b->ctx) hist[{c->kind, c->L}] += 1;
+    // signature of the batch for the tuning cache: SM count, sweeps, and the items
+    // of the launch that is tuned, by class
     b->sig = std::to_string(sms) + "|" + std::to_string(n_sweeps);
-    for (auto& kv : hist)
-        b->sig += "|" + std::to_string(kv.first.first) + ":" + std::to_string(kv.first.second) + "x" +
-                  std::to_string(kv.second);
+    for (auto& kv : tuned_items) b->sig += "|" + std::to_string(kv.first) + "x" + std::to_string(kv.second);
     if (b->tune_mode == 0) {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(b->sig);
@@ -1890,6 +1889,7 @@ static int batch_tune(pa_batch* b, int k)
     b->tuned_ms = best;
     b->tuned = true;
     std::lock_guard<std::mutex> lk(g_tune_mu);
+    if (g_tune_cache.size() >= 1024) g_tune_cache.clear();
     g_tune_cache[b->sig] = {bb, bm};
     return PA_OK;
 }

@@ -166,3 +166,25 @@ def test_an_anneal_without_eager_steps_is_all_or_nothing(fake, call, after):
         assert P.pa_current_step(ctx) == 9 and len(f.launched("observe_kernel")) == 9
     finally:
         P.pa_destroy(ctx)
+
+
+@pytest.mark.parametrize("first,second", [
+    # +-J beside real couplings with and without a field: per-attempt tiles, or the table launch
+    ([(0, 4, 7000, False), (1, 10, 300, True)], [(0, 4, 7000, False), (1, 10, 300, False)]),
+    # the same lattices with other populations: other lists of items
+    ([(0, 6, 300, False), (0, 8, 300, False)], [(0, 6, 90_000, False), (0, 8, 300, False)]),
+])
+def test_batches_with_other_items_are_tuned_on_their_own(fake, first, second):
+    P, f = fake
+    tunings = []
+    for insts in (first, second, first):
+        b = _batch(P, insts)
+        try:
+            P.pa_batch_run(b, 1)
+            f.reset()
+            P.pa_batch_run(b, 1)  # the first step that can be tuned
+            tunings.append(len(f.launched("sweep_batch_kernel")) > 1)
+            assert (P.pa_batch_sweep_config(b)["tuned_ms"] > 0) == tunings[-1]
+        finally:
+            P.pa_batch_destroy(b)
+    assert tunings == [True, True, False]  # the third takes the first one's shape
