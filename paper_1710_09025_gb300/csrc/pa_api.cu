@@ -1742,16 +1742,16 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
         }
         c->k_next = 0; c->cur = 0; c->famcur = 0;
     }
-    // chunks of the threshold-table launch: as large as leaves two per SM (a
-    // chunk builds the instance's table, so small ones cost work; too few leave
-    // SMs idle)
+    // chunks of the threshold-table launch: as large as leaves that launch two per
+    // SM (a chunk builds the instance's table, so small ones cost work; too few
+    // leave SMs idle)
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     for (; b->tchunk > pa::kBatchTableLeast; b->tchunk /= 2) {
         long long n = 0;
-        for (auto* c : b->ctx)
-            if (c->kind == PA_REAL) n += ((c->R + 3) / 4 + b->tchunk - 1) / b->tchunk;
+        for (int i = 0; i < n_inst; ++i)
+            if (sw[i].cls >= pa::kBatchTableBase) n += ((b->ctx[i]->R + 3) / 4 + b->tchunk - 1) / b->tchunk;
         if (n >= 2ll * sms) break;
     }
     // work items, most expensive first (estimated thread-instructions per
@@ -1772,7 +1772,8 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
             smax = std::max(smax, sm);
             int gpb = 0, thr = 0;
             pa::packed_default_shape(D, c->L, &gpb, &thr);
-            double cost = c->kind == PA_PM1 ? (double)gpb * m * c->N * 700.0 : 32.0 * c->N * 70.0;
+            const double real = m == 0 ? (double)c->R / tiles : 32.0;  // replicas of an item
+            double cost = c->kind == PA_PM1 ? (double)gpb * m * c->N * 700.0 : real * c->N * 70.0;
             for (int t = 0; t < tiles; ++t) items.push_back({cost, i, t});
         }
         std::stable_sort(items.begin(), items.end(), [](const It& x, const It& y) { return x.cost > y.cost; });

@@ -188,3 +188,36 @@ def test_batches_with_other_items_are_tuned_on_their_own(fake, first, second):
         finally:
             P.pa_batch_destroy(b)
     assert tunings == [True, True, False]  # the third takes the first one's shape
+
+
+def _table_launch(P, f, insts):
+    """(chunk, items) of a batch's threshold-table launch"""
+    b = _batch(P, insts, threads=-1)
+    try:
+        assert P.pa_batch_step(b)
+        items = np.zeros((f.lib.fake_table_items(None, 0), 2), np.int32)
+        f.lib.fake_table_items(items.ctypes.data_as(ctypes.c_void_p), items.size)
+        return f.lib.fake_table_chunk(), items
+    finally:
+        P.pa_batch_destroy(b)
+
+
+@pytest.mark.parametrize("others", [[(1, 12, 60_000, False)], [(1, 10, 60_000, True)], [(0, 8, 60_000, False)]])
+def test_chunks_go_by_the_instances_of_the_table_launch(fake, others):
+    P, f = fake
+    alone, items = _table_launch(P, f, [(1, 4, 8000, False)])
+    assert alone == 8 and len(items) == 250  # 2000 groups: fewer than two chunks per SM even of the smallest
+    chunk, beside = _table_launch(P, f, [(1, 4, 8000, False)] + others)
+    assert chunk == alone
+    np.testing.assert_array_equal(beside, items)
+
+
+def test_table_items_come_by_cost(fake):
+    """The most expensive first: sites times replicas of the chunk."""
+    P, f = fake
+    insts = [(1, 8, 40, False), (1, 6, 120_000, False), (1, 4, 90_000, True), (1, 10, 12, False)]
+    chunk, items = _table_launch(P, f, insts)
+    n = [len(items[items[:, 0] == i]) for i in range(len(insts))]
+    assert n == [-(-((R + 3) // 4) // chunk) for _, _, R, _ in insts]
+    cost = [insts[i][1] ** 3 * insts[i][2] / n[i] for i in items[:, 0]]
+    assert cost == sorted(cost, reverse=True)
