@@ -1918,26 +1918,32 @@ static int batch_enqueue(pa_batch* b, bool allow_tune)
     batch_step_params(b, k, &ps, &rs);
     const pa::BatchSweepInst* tab = b->d_sw + (size_t)k * b->n_inst;
     // the two sweep launches are independent: the threshold-table one runs on
-    // the batch's second stream between two events
-    cudaStream_t ts = b->st2 ? b->st2 : b->st;
+    // the batch's second stream between two events.  The join is made whatever the
+    // other launch returns, so that nothing enqueued later on the batch's stream
+    // can run beside a table launch that was under way.
+    cudaError_t es = cudaSuccess;
     if (b->n_titems > 0) {
+        cudaStream_t ts = b->st2 ? b->st2 : b->st;
         if (b->st2) {
             PB_CK(b, cudaEventRecord(b->ev_fork, b->st));
             PB_CK(b, cudaStreamWaitEvent(b->st2, b->ev_fork, 0));
         }
-        PB_CK(b, pa::launch_sweep_batched_table(rs, tab, b->d_titems, b->n_titems, b->tchunk,
-                                                b->d_counters + b->n_temps + kTuneSlots + k, b->tblocks, b->tsmem,
-                                                ts));
+        es = pa::launch_sweep_batched_table(rs, tab, b->d_titems, b->n_titems, b->tchunk,
+                                            b->d_counters + b->n_temps + kTuneSlots + k, b->tblocks, b->tsmem, ts);
         b->launches += 1;
     }
-    if (b->n_items[b->mult - 1] > 0) {
-        PB_CK(b, pa::launch_sweep_batched(ps, rs, tab, b->d_items[b->mult - 1], b->n_items[b->mult - 1], b->mult,
-                                          b->d_counters + k, b->blocks, b->smem[b->mult - 1], b->st));
+    if (es == cudaSuccess && b->n_items[b->mult - 1] > 0) {
+        es = pa::launch_sweep_batched(ps, rs, tab, b->d_items[b->mult - 1], b->n_items[b->mult - 1], b->mult,
+                                      b->d_counters + k, b->blocks, b->smem[b->mult - 1], b->st);
         b->launches += 1;
     }
     if (b->st2 && b->n_titems > 0) {
-        PB_CK(b, cudaEventRecord(b->ev_join, b->st2));
-        PB_CK(b, cudaStreamWaitEvent(b->st, b->ev_join, 0));
+        const cudaError_t er = cudaEventRecord(b->ev_join, b->st2), ew = cudaStreamWaitEvent(b->st, b->ev_join, 0);
+        if (es == cudaSuccess) es = er != cudaSuccess ? er : ew;
+    }
+    if (es != cudaSuccess) {
+        b->err = std::string("batched sweeps: ") + cudaGetErrorString(es);
+        return PA_ECUDA;
     }
     PB_CK(b, pa::launch_observe_batched(b->d_ob + (size_t)k * b->n_inst, b->n_inst, b->maxR, b->st));
     b->launches += 1;

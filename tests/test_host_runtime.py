@@ -221,3 +221,31 @@ def test_table_items_come_by_cost(fake):
     assert n == [-(-((R + 3) // 4) // chunk) for _, _, R, _ in insts]
     cost = [insts[i][1] ** 3 * insts[i][2] / n[i] for i in items[:, 0]]
     assert cost == sorted(cost, reverse=True)
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_an_error_beside_the_table_launch_still_joins_it(fake, graph):
+    """What follows on the batch's stream waits for the second stream's launch."""
+    P, f = fake
+    b = _batch(P, [(0, 4, 300, False), (1, 4, 300, False)], n=5, threads=-1)
+    try:
+        P.pa_batch_run(b, 2)
+        f.reset()
+        f.fail("sweep_batch_kernel")
+        with pytest.raises(P.PAError):
+            P.pa_batch_run(b, -1) if graph else P.pa_batch_step(b)
+        assert P.pa_batch_current_step(b) == 2
+        if graph:  # nothing of the capture runs
+            assert not f.launched("")
+        else:
+            log = f.log()
+            at = next(i for i, x in enumerate(log) if "sweep_batch_table_kernel" in x)
+            side = log[at].split(" stream ")[1].split()[0]
+            assert side != str(STREAM)
+            assert log[at + 1].startswith("record ") and log[at + 1].endswith(" stream " + side)
+            event = log[at + 1].split()[1]
+            assert log[at + 2] == f"wait {event} stream {STREAM}"
+        P.pa_batch_run(b, -1)
+        assert P.pa_batch_current_step(b) == 5
+    finally:
+        P.pa_batch_destroy(b)
