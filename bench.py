@@ -307,7 +307,7 @@ def run_gpu(args, wl_name):
                      "algorithmic_bytes_per_launch": bytes_launch,
                      "note": "per-sweep streaming bytes per attempted flip (spin read + written "
                              "each sweep); the kernel keeps the state in shared memory for all N_S "
-                             "sweeps and is bound by integer ALU issue, not DRAM",
+                             "sweeps and is bound by integer work on the SMs, not DRAM",
                      # the binding unit, from the committed ncu record of this kernel source
                      "alu_pipe_of_peak_ncu": rec.get("alu_pipe_of_peak") if rec else None},
         "phases_ms_per_step": per_step,

@@ -41,7 +41,7 @@ struct pa_ctx {
     int scheme;                 // PA_RESAMPLE_*; nearest-integer: populations in Rdev
     int icm;                    // isoenergetic cluster moves and their beta window
     double icm_lo, icm_hi;
-    int* icm_err;               // device flag: a bounded union-find loop gave up
+    int* icm_err;               // device flag: an island did not close within its bound
     double *runP, *runq;        // resampling: run table
     int32_t* bcount;            // resampling: copies per scan block
     int* sync;                  // block counters of the merged launches (zeroed)
@@ -1011,7 +1011,7 @@ extern "C" int pa_synchronize(pa_ctx* c)
     if (c->icm) {
         int bad = 0;
         PA_CK(c, cudaMemcpy(&bad, c->icm_err, sizeof(int), cudaMemcpyDeviceToHost));
-        if (bad) { c->err = "a cluster-move union-find loop reached its bound"; return PA_ETIMEOUT; }
+        if (bad) { c->err = "the island of a cluster move did not close within its bound"; return PA_ETIMEOUT; }
     }
     int R;
     return pop_now(c, &R);  // PA_EEMPTY once the population died out

@@ -11,9 +11,10 @@
 // the spins of that site's island are flipped in both replicas.  With a zero
 // field E_a + E_b is unchanged, so the move is always accepted.
 //
-// Four launches: both rounds' pairings (one thread per replica) with the packed
-// words turned into one bit row per replica; two rounds of moves, one warp per
-// pair; the rows turned back.  A pair then reads N / 8 bytes per replica instead
+// Five launches with packed words (three with int8 rows, which need no turning):
+// both rounds' pairings, one thread per replica; the words turned into one bit row
+// per replica; two rounds of moves, one warp per pair; the rows turned back.  A
+// pair then reads N / 8 bytes per replica instead
 // of a 64-bit word per site, and its island grows by whole x-rows: the sector and
 // the island are L-bit rows in shared memory, a row takes the bits next to the
 // rows around it and fills the sector's runs that touch them with one addition

@@ -125,8 +125,8 @@ cudaError_t launch_overlap_i8(const int8_t* A, const int8_t* B, int N, int NP, i
 // ---------------- batched sweep ----------------
 constexpr int kBatchRealBase = 100;   // class ids >= this are real-coupling tiles
 constexpr int kBatchTableBase = 200;  // class ids >= this are threshold-table chunks (their own launch)
-constexpr int kBatchTableGroups = 64; // most and fewest replica groups (of four) per chunk
-constexpr int kBatchTableLeast = 8;
+constexpr int kBatchTableGroups = 64; // most replica groups (of four) per chunk
+constexpr int kBatchTableLeast = 8;   // and the size below which chunks are not halved any more
 struct BatchSweepInst {
     int cls;                 // packed: 2 * lattice index (+1 for the doubled groups per block)
     int pad;
@@ -154,7 +154,7 @@ struct IcmArgs {
     int* perm;               // [2][R] scratch: both rounds' pairings
     uint32_t* rows;          // packed words: [R][(N + 31) / 32] scratch, a bit row per replica
     uint32_t key0, key1, c3; // Philox key, counter word 3 of the ICM stream
-    int* err;                // set if a bounded union-find loop gave up
+    int* err;                // set if an island did not close within its bound
 };
 cudaError_t launch_icm(const IcmArgs& a, int* launches, cudaStream_t st);
 

@@ -16,9 +16,10 @@
 // the products with the last neighbour's sign matter (IEEE sums of negated
 // terms are the negated sums), which halves the patterns.
 //
-// What bounds it: integer instructions, two cycles each on an SM quarter
-// whether they multiply or not (ncu: ALU plus multiply instructions times two
-// account for every cycle).  A Philox call serves four attempts (the WORD
+// What bounds it: integer instructions, of which the ALU takes more than the
+// multiplier; no unit is full (ncu at 3D L = 10: ALU pipe 64 % of its cycles,
+// multiplier 53 %, issue slots 59 %; 384 to 1024 threads a block within 5 %), but
+// the time has followed their number.  A Philox call serves four attempts (the WORD
 // stream: the four sites of a quad, one replica) with 34 of them; four replicas
 // of a quad take about 285, 18 per attempt.  Field, exponential and guard band
 // per attempt took 86.  Gaussian couplings, N_S = 10, sweep time per

@@ -9,6 +9,7 @@ import pytest
 
 from paper_1710_09025_gb300 import workloads as W
 from test_gpu_batch import PM1, REAL, _snapshot
+from test_gpu_parity import run_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -50,3 +51,12 @@ def test_batch_tiles_with_the_specified_rule_match(pa):
         for g, w in zip(got[:5], want[:5]):
             np.testing.assert_array_equal(g, w)
         assert got[5] == want[5]
+
+
+@pytest.mark.parametrize("L,field,R,threads", [(12, True, 333, 0), (12, False, 97, 128), (10, True, 250, 0)])
+def test_tiles_match_the_oracle(pa, oracle, L, field, R, threads):
+    """Several tiles of 32 replicas and a ragged last one, gradient counts included."""
+    J = W.couplings_gauss(3, L, 61 + L)
+    h = W.field_uniform(L ** 3, 62 + L) if field else None
+    pop, _ = run_parity(pa, oracle, 3, L, REAL, J, h, R, W.schedule_lb(4, 4.0), 2, 63 + L, grad=True, threads=threads)
+    pop.close()
