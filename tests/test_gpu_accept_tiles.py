@@ -9,7 +9,6 @@ import pytest
 
 from paper_1710_09025_gb300 import workloads as W
 from test_gpu_batch import PM1, REAL, _snapshot
-from test_gpu_parity import run_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -55,8 +54,24 @@ def test_batch_tiles_with_the_specified_rule_match(pa):
 
 @pytest.mark.parametrize("L,field,R,threads", [(12, True, 333, 0), (12, False, 97, 128), (10, True, 250, 0)])
 def test_tiles_match_the_oracle(pa, oracle, L, field, R, threads):
-    """Several tiles of 32 replicas and a ragged last one, gradient counts included."""
+    """Several tiles of 32 replicas and a ragged last one: what the sweeps produce
+    (spins, int128 energies, gradient counts) and the parents that follow from it,
+    bit for bit."""
+    P = pa
     J = W.couplings_gauss(3, L, 61 + L)
     h = W.field_uniform(L ** 3, 62 + L) if field else None
-    pop, _ = run_parity(pa, oracle, 3, L, REAL, J, h, R, W.schedule_lb(4, 4.0), 2, 63 + L, grad=True, threads=threads)
-    pop.close()
+    betas = W.schedule_lb(4, 4.0)
+    ref = oracle.Sim(3, L, REAL, J, h, R, betas, 2, 63 + L, accumulate_grad=True)
+    pop = P.Population(3, L, REAL, J, h, R, betas, 2, 63 + L, accumulate_grad=1, threads=threads)
+    try:
+        for k in range(len(betas)):
+            assert pop.step()
+            ref.step()
+            np.testing.assert_array_equal(P.pa_get_spins(pop.ctx), ref.spins(), err_msg=f"spins k={k}")
+            np.testing.assert_array_equal(P.pa_get_energies(pop.ctx, REAL), ref.energies_raw(), err_msg=f"E k={k}")
+            if k > 0:
+                np.testing.assert_array_equal(P.pa_get_parents(pop.ctx), ref.parents(), err_msg=f"parents k={k}")
+        for got, want in zip(P.pa_get_grad_counts(pop.ctx), ref.grad_counts()):
+            np.testing.assert_array_equal(got, want)
+    finally:
+        pop.close()
