@@ -1568,8 +1568,10 @@ extern "C" void pa_destroy(pa_ctx* c)
 // observables for all instances.
 
 #include <algorithm>
+#include <functional>
 #include <map>
 #include <mutex>
+#include <queue>
 
 struct pa_batch {
     int D, n_inst, n_temps, n_sweeps, k_next;
@@ -1744,16 +1746,48 @@ extern "C" int pa_batch_create(pa_batch** out, int D, int n_inst, const pa_inst_
     }
     // chunks of the threshold-table launch: as large as leaves that launch two per
     // SM (a chunk builds the instance's table, so small ones cost work; too few
-    // leave SMs idle)
+    // leave SMs idle), or else the smallest ones of which no SM gets a second, where
+    // the queue would be done earlier with these.  Sweeps of 12 temperatures, two
+    // per SM -> one per SM: 3D L=4 with a field 8 x R=2000 1520 -> 877 us (per-attempt
+    // tiles 1310), 16 x R=2000 1550 -> 1011; without a field L=8 16 x R=2000 3140 ->
+    // 2716, L=10 8 x R=2000 3725 -> 2955, L=10 R=10000 2943 -> 2971.
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    for (; b->tchunk > pa::kBatchTableLeast; b->tchunk /= 2) {
+    auto chunks_of = [&](int i, int chunk) {
+        return sw[i].cls >= pa::kBatchTableBase ? ((b->ctx[i]->R + 3) / 4 + chunk - 1) / chunk : 0;
+    };
+    auto count = [&](int chunk) {
         long long n = 0;
-        for (int i = 0; i < n_inst; ++i)
-            if (sw[i].cls >= pa::kBatchTableBase) n += ((b->ctx[i]->R + 3) / 4 + b->tchunk - 1) / b->tchunk;
-        if (n >= 2ll * sms) break;
-    }
+        for (int i = 0; i < n_inst; ++i) n += chunks_of(i, chunk);
+        return n;
+    };
+    // when the queue is done, an item at a time per SM, in sites times replica groups:
+    // a table costs about 5 groups' sweeps (9 with a field), and a chunk cannot take
+    // less than one group per slot of the block's threads
+    auto done_at = [&](int chunk) {
+        std::vector<double> cost;
+        for (int i = 0; i < n_inst; ++i) {
+            const int n = chunks_of(i, chunk), N = b->ctx[i]->N;
+            const double groups = n ? (b->ctx[i]->R + 3) / 4 / (double)n : 0.0;
+            cost.insert(cost.end(), n, N * ((b->ctx[i]->field ? 9.0 : 5.0) + std::max(groups, 4096.0 / N)));
+        }
+        std::sort(cost.begin(), cost.end(), std::greater<double>());
+        std::priority_queue<double, std::vector<double>, std::greater<double>> free_at(
+            std::greater<double>(), std::vector<double>(std::max(sms, 1), 0.0));
+        double last = 0.0;
+        for (double c : cost) {
+            const double t = free_at.top() + c;
+            free_at.pop();
+            free_at.push(t);
+            last = std::max(last, t);
+        }
+        return last;
+    };
+    while (b->tchunk > pa::kBatchTableLeast && count(b->tchunk) < 2ll * sms) b->tchunk /= 2;
+    int one = pa::kBatchTableLeast;
+    while (one < pa::kBatchTableGroups && count(one) > sms) one *= 2;
+    if (one > b->tchunk && count(one) <= sms && done_at(one) < done_at(b->tchunk)) b->tchunk = one;
     // work items, most expensive first (estimated thread-instructions per
     // tile): one list for the launch of each groups-per-block multiplier, one
     // (m = 0) for the threshold-table launch

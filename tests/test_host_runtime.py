@@ -206,7 +206,7 @@ def _table_launch(P, f, insts):
 def test_chunks_go_by_the_instances_of_the_table_launch(fake, others):
     P, f = fake
     alone, items = _table_launch(P, f, [(1, 4, 8000, False)])
-    assert alone == 8 and len(items) == 250  # 2000 groups: fewer than two chunks per SM even of the smallest
+    assert alone == 16 and len(items) == 125  # 2000 groups
     chunk, beside = _table_launch(P, f, [(1, 4, 8000, False)] + others)
     assert chunk == alone
     np.testing.assert_array_equal(beside, items)
@@ -249,3 +249,18 @@ def test_an_error_beside_the_table_launch_still_joins_it(fake, graph):
         assert P.pa_batch_current_step(b) == 5
     finally:
         P.pa_batch_destroy(b)
+
+
+@pytest.mark.parametrize("insts,chunk,items", [
+    ([(1, 4, 2000, True)] * 8, 32, 128),      # one chunk per SM at most, instead of three or four small ones
+    ([(1, 10, 2000, False)] * 8, 32, 128),
+    ([(1, 8, 1000, False)] * 32, 64, 128),
+    ([(1, 4, 200, True)] * 32, 16, 128),
+    ([(1, 10, 2000, False)], 8, 63),          # the smallest already leave no SM a second one
+    ([(1, 10, 40_000, False)], 32, 313),      # more than the largest chunks on every SM: two per SM
+    ([(1, L, 2000, False) for L in (4, 6, 8, 10)], 8, 252),  # the largest lattice's chunks would be the last
+])
+def test_a_chunk_per_sm_where_the_queue_is_done_earlier(fake, insts, chunk, items):
+    P, f = fake
+    got, queue = _table_launch(P, f, insts)
+    assert (got, len(queue)) == (chunk, items)
